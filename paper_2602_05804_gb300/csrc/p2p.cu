@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "fexp.cuh"
 #include "sfmm_internal.cuh"
 
 namespace sfmm {
@@ -60,6 +61,7 @@ struct P2PArgs {
   int lmax;
   int chunk;          // neighbour-list entries per work item of a split list
   unsigned long long* pair_counter;  // pair evaluations (statistics)
+  const int* items;   // FP64 form: the work items k_p2p_fexp left, items[-4] of them
 };
 
 // M4 softening kernel of one particle (compact support 2h): g = phi'(r)/r
@@ -178,6 +180,8 @@ __device__ __forceinline__ void p2p_finish(const P2PArgs& a, int i, const R (&v)
   if (a.pot) a.pot[o] = pot;
 }
 
+#include "p2p_fexp.cuh"
+
 // One warp per target leaf.  Sources: the particles of the leaf's neighbour
 // list, streamed 32 at a time over consecutive list entries (every lane
 // busy), moved to the target leaf's frame (FP32 form) and split once per
@@ -202,13 +206,14 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = lanemask_lt();
   const int nextra = (int)a.d_split[0];
-  const int nitems = nextra + (int)a.counts[1];
+  const int nitems = F32 ? nextra + (int)a.counts[1] : a.items[-4];
   unsigned long long pairs = 0;  // this lane's share of the pair evaluations
   while (true) {
     int item = 0;
     if (lane == 0) item = atomicAdd(a.leaf_counter, 1);
     item = __shfl_sync(SFMM_FULL, item, 0);
     if (item >= nitems) break;
+    if constexpr (!F32) item = a.items[item];
     int leaf, chunk = 0;
     if (item < nextra) {
       const int2 x = a.extra[item];
@@ -767,8 +772,38 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   if (per_sm < 1) per_sm = 1;
   if (c->p2p_blocks > 0 && c->p2p_blocks < per_sm) per_sm = c->p2p_blocks;  // option: fewer blocks per SM
   const int nblocks = per_sm * num_sms(c->device);
-  if (f32) k_p2p<true><<<nblocks, nt, 0, c->stream>>>(a);
-  else k_p2p<false><<<nblocks, nt, 0, c->stream>>>(a);
+  if (f32) {
+    k_p2p<true><<<nblocks, nt, 0, c->stream>>>(a);
+  } else {
+    // FP32-pipe expansions first; what they cannot take (usually nothing)
+    // is left to the FP64 kernel
+    const size_t n = (size_t)c->n;
+    if ((rc = c->fx_rec.ensure((3 * sizeof(float4) + sizeof(float2) + sizeof(double)) * n)) ||
+        (rc = c->fx_items.ensure(sizeof(int) * (4 + (size_t)nl_b + (size_t)nextra))))
+      return rc;
+    FexpArgs f{};
+    f.psys = c->nsys > 1 ? c->psys.as<int>() : nullptr;
+    f.sys_root = c->sys_root.as<int>();
+    f.nsize = c->nsize.as<double>();
+    f.nmass = c->nmass.as<double>();
+    f.rec0 = c->fx_rec.as<float4>();
+    f.rec1 = f.rec0 + n;
+    f.rec2 = f.rec1 + n;
+    f.rech = reinterpret_cast<float2*>(f.rec2 + n);
+    f.hinv = reinterpret_cast<double*>(f.rech + n);
+    f.fb = c->fx_items.as<int>();
+    k_fexp_records<<<(int)std::min<size_t>((n + 255) / 256, 8 * (size_t)num_sms(c->device)), 256, 0, c->stream>>>(
+        a, f, (int)n);
+    int fx_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fx_sm, k_p2p_fexp, FX_NT, 0);
+    fx_sm = std::max(1, fx_sm);
+    if (c->p2p_blocks > 0 && c->p2p_blocks < fx_sm) fx_sm = c->p2p_blocks;
+    k_p2p_fexp<<<fx_sm * num_sms(c->device), FX_NT, 0, c->stream>>>(a, f);
+    a.leaf_counter = f.fb + 1;
+    a.items = f.fb + 4;
+    k_p2p<false><<<nblocks, nt, 0, c->stream>>>(a);
+    c->nlaunch += 2;
+  }
   ++c->nlaunch;
   SFMM_CUDA_TRY(cudaGetLastError());
   {
@@ -784,10 +819,10 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
 
 int p2p_blocks_fit(sfmm_ctx* c) {
   const bool f32 = (c->precision == SFMM_FP32);
-  const int nt = 32 * (f32 ? p2p_warps<true>() : p2p_warps<false>());
+  const int nt = 32 * p2p_warps<true>();
   int per_sm = 0;
   if (f32) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<true>, nt, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<false>, nt, 0);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_fexp, FX_NT, 0);
   return per_sm < 1 ? 1 : per_sm;
 }
 

@@ -116,6 +116,7 @@ struct sfmm_ctx {
   // near field: chunks of long neighbour lists (extra work items, per-leaf
   // slot base, split leaves, partial sums) and the list entries in use
   DevBuf p2p_extra, p2p_split, p2p_slist, p2p_part;
+  DevBuf fx_rec, fx_items;  // FP64 form: particle records as float expansions, items left to the FP64 kernel
   // leapfrog: accelerations, per-tile momentum partials and their sum
   DevBuf lf_acc, lf_part;
   // kd-tree build: particle orders, breadth-first node records, level scratch
