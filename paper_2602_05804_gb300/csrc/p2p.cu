@@ -778,7 +778,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
     // FP32-pipe expansions first; what they cannot take (usually nothing)
     // is left to the FP64 kernel
     const size_t n = (size_t)c->n;
-    if ((rc = c->fx_rec.ensure((3 * sizeof(float4) + sizeof(float2) + sizeof(double)) * n)) ||
+    if ((rc = c->fx_rec.ensure((3 * sizeof(float4) + sizeof(float2) + sizeof(double2)) * n + 16)) ||
         (rc = c->fx_items.ensure(sizeof(int) * (4 + (size_t)nl_b + (size_t)nextra))))
       return rc;
     FexpArgs f{};
@@ -789,8 +789,8 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
     f.rec0 = c->fx_rec.as<float4>();
     f.rec1 = f.rec0 + n;
     f.rec2 = f.rec1 + n;
-    f.rech = reinterpret_cast<float2*>(f.rec2 + n);
-    f.hinv = reinterpret_cast<double*>(f.rech + n);
+    f.hinv = reinterpret_cast<double2*>(f.rec2 + n);
+    f.rech = reinterpret_cast<float2*>(f.hinv + n);
     f.fb = c->fx_items.as<int>();
     k_fexp_records<<<(int)std::min<size_t>((n + 255) / 256, 8 * (size_t)num_sms(c->device)), 256, 0, c->stream>>>(
         a, f, (int)n);

@@ -29,7 +29,7 @@ struct FexpArgs {
   float4* rec1;         // {x, y, z (grid 2^-45), m (next 24)}
   float4* rec2;         // {x, y, z (rest), m (rest)}
   float2* rech;         // {(2h)^2 rounded up, 2h rounded down}, scaled
-  double* hinv;         // 1 / h
+  double2* hinv;        // {1 / h, 1 / h^3}
   int* fb;              // [0] work items left to k_p2p<false>, [1] its item counter, [4 ..] the items
 };
 
@@ -46,7 +46,8 @@ __device__ __forceinline__ SysScale sys_scale(const P2PArgs& a, const FexpArgs& 
 __global__ void __launch_bounds__(256) k_fexp_records(const P2PArgs a, const FexpArgs f, int n) {
   if (blockIdx.x == 0 && threadIdx.x < 4) f.fb[threadIdx.x] = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    f.hinv[i] = 1.0 / a.ph[i];
+    const double hi = 1.0 / a.ph[i];
+    f.hinv[i] = make_double2(hi, hi * hi * hi);
     const SysScale s = sys_scale(a, f, i);
     if (!s.ok) continue;  // (not read: every leaf of the system goes to k_p2p<false>)
     const double sx = __hiloint2double((1023 - s.kx) << 20, 0), sm = __hiloint2double((1023 - s.km) << 20, 0);
@@ -63,23 +64,42 @@ __global__ void __launch_bounds__(256) k_fexp_records(const P2PArgs a, const Fex
   }
 }
 
-// M4 kernel of one particle in FP64, piece chosen by its coefficients (an FP64
-// instruction takes the time of many selects): g and phi of a unit mass at r = q h, summed
-// into g, phi.
-__device__ __forceinline__ void m4_add(double r, double ri, double ri3, double hinv, double& g, double& phi) {
-  const double q = r * hinv;
-  const bool in1 = q < 1.0, out = q >= 2.0;
+// 1 / sqrt(x) to about an ulp in three FP64 instructions where the library
+// takes ten: the FP32 estimate y with its FP64 remainder e = 1 - x y^2
+// (|e| < 2^-20), y (1 + e/2 + 3/8 e^2) with the last term (below 2^-41)
+// formed in FP32 and placed in the 29 low bits that y leaves free, and the
+// conversions done on the bit patterns.  x in [2^-120, 2^120].
+__device__ __forceinline__ double rsqrt_refined(double x) {
+  const unsigned hi = __double2hiint(x), lo = __double2loint(x);
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29))));
+  const unsigned yb = __float_as_uint(y);
+  const unsigned yh = (yb >> 3) + 0x38000000u, yl = yb << 29;
+  const double yd = __hiloint2double(yh, yl);
+  const double e = ::fma(-(x * yd), yd, 1.0);
+  const float ef = __int_as_float(max((__double2hiint(e) & 0x7fffffff) - 0x38000000, 0) << 3);
+  const float k = (0.375f * 0x1p52f) * (ef * ef) * __uint_as_float((yb & 0x7fffffu) | 0x3f800000u);
+  const unsigned n = __float_as_uint(k + 8388608.0f) & 0x7fffffu;  // k rounded to an integer (< 2^12)
+  return ::fma(__hiloint2double(yh - 0x100000u, yl), e, __hiloint2double(yh, yl + n));
+}
+
+// M4 kernel of one particle in FP64: g and phi of a unit mass at r = q h,
+// added to g, phi.  The piece is chosen by its coefficients (an FP64
+// instruction takes the time of many selects) and by integer comparison.
+__device__ __forceinline__ void m4_add(double r, double ri, double ri3, double2 hinv, double& g, double& phi) {
+  const double q = r * hinv.x;
+  const int qh = __double2hiint(q);
+  const bool in1 = qh < 0x3ff00000, out = qh >= 0x40000000;  // q < 1, q >= 2
   const double g0 = in1 ? 4.0 / 3.0 : 8.0 / 3.0, g1 = in1 ? 0.0 : -3.0, g2 = in1 ? -1.2 : 1.2,
                g3 = in1 ? 0.5 : -1.0 / 6.0;
   const double p0 = in1 ? -1.4 : -1.6, p2 = in1 ? 2.0 / 3.0 : 4.0 / 3.0, p3 = in1 ? 0.0 : -1.0,
                p4 = in1 ? -0.3 : 0.3, p5 = in1 ? 0.1 : -1.0 / 30.0;
   // outside 2h the polynomials take no part: 1/r^3 and -1/r
-  const double hv = out ? 0.0 : hinv, qq = out ? 0.0 : q;
+  const double hv = out ? 0.0 : hinv.x, hv3 = out ? 0.0 : hinv.y, qq = out ? 0.0 : q;
   const double cg = in1 ? 0.0 : (out ? 1.0 : -1.0 / 15.0), cp = in1 ? 0.0 : (out ? -1.0 : 1.0 / 15.0);
-  const double q2 = qq * qq;
   const double gp = ::fma(qq, ::fma(qq, ::fma(qq, g3, g2), g1), g0);
-  const double pp = ::fma(q2, ::fma(qq, ::fma(qq, ::fma(qq, p5, p4), p3), p2), p0);
-  g = ::fma(hv * hv * hv, gp, ::fma(cg, ri3, g));
+  const double pp = ::fma(qq * qq, ::fma(qq, ::fma(qq, ::fma(qq, p5, p4), p3), p2), p0);
+  g = ::fma(hv3, gp, ::fma(cg, ri3, g));
   phi = ::fma(hv, pp, ::fma(cp, ri, phi));
 }
 
@@ -104,7 +124,8 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
   __shared__ int s_idx[FX_WARPS][FX_SB + 2];
   __shared__ double s_acc[FX_WARPS][64][4];
   __shared__ __align__(16) float s_part[FX_WARPS][12][32];  // run sums; softened results (32 x 4 doubles)
-  __shared__ unsigned short s_sq[FX_WARPS][FX_SQ];
+  __shared__ int s_qj[FX_WARPS][FX_SQ];  // queued softened pairs: source particle, target in the leaf
+  __shared__ unsigned char s_qt[FX_WARPS][FX_SQ];
   __shared__ float2 s_bias[FX_WARPS][32];  // per target of a group: level-0 bias of force and potential
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -170,19 +191,20 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
     // lane of each target adds the target's results in lane order
     auto soft_batch = [&](int base, int nb) {
       double4_16a* const res = reinterpret_cast<double4_16a*>(&s_part[warp][0][0]);
-      const int ent = lane < nb ? (int)s_sq[warp][base + lane] : 0;
-      const int t = lane < nb ? ent >> 8 : 64 + lane;
+      const int t = lane < nb ? (int)s_qt[warp][base + lane] : 64 + lane;
       double4_16a v = make_double4_16a(0.0, 0.0, 0.0, 0.0);
       if (lane < nb) {
-        const int i = fL + t, j = s_idx[warp][ent & 255];
+        const int i = fL + t, j = s_qj[warp][base + lane];
         const double dx = a.px[i] - a.px[j], dy = a.py[i] - a.py[j], dz = a.pz[i] - a.pz[j];
         const double r2 = ::fma(dx, dx, ::fma(dy, dy, dz * dz));
-        const double ri = r2 > 0.0 ? rsqrt(r2) : 0.0;
+        // (coincident particles: no force, the kernel's central potential)
+        const double ri = (r2 >= 0x1p-120 && r2 <= 0x1p120) ? rsqrt_refined(r2) : (r2 > 0.0 ? rsqrt(r2) : 0.0);
         const double r = r2 * ri, ri3 = ri * ri * ri;
         double g = 0.0, phi = 0.0;
         m4_add(r, ri, ri3, f.hinv[i], g, phi);
         m4_add(r, ri, ri3, f.hinv[j], g, phi);
-        const double mh = 0.5 * a.pm[j], mg = -mh * g;
+        const double mj = a.pm[j], mh = __hiloint2double(__double2hiint(mj) - 0x100000, __double2loint(mj));
+        const double mg = -mh * g;
         v = make_double4_16a(mg * dx, mg * dy, mg * dz, mh * phi);
       }
       const unsigned same = __match_any_sync(SFMM_FULL, t);
@@ -404,9 +426,16 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
           }
           const unsigned bx = __ballot_sync(SFMM_FULL, inx), by = __ballot_sync(SFMM_FULL, iny);
           if (bx | by) {
-            const int slot = ((g0 + t) << 8) | (2 * j);
-            if (inx) s_sq[warp][qn + __popc(bx & lt)] = (unsigned short)slot;
-            if (iny) s_sq[warp][qn + __popc(bx) + __popc(by & lt)] = (unsigned short)(slot + 1);
+            if (inx) {
+              const int w = qn + __popc(bx & lt);
+              s_qj[warp][w] = s_idx[warp][2 * j];
+              s_qt[warp][w] = (unsigned char)(g0 + t);
+            }
+            if (iny) {
+              const int w = qn + __popc(bx) + __popc(by & lt);
+              s_qj[warp][w] = s_idx[warp][2 * j + 1];
+              s_qt[warp][w] = (unsigned char)(g0 + t);
+            }
             qn += __popc(bx) + __popc(by);
             __syncwarp();
             while (qn >= 32) {
@@ -454,14 +483,10 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
         }
         __syncwarp();
       }
-      // the queue refers to staged sources: empty it before they are replaced
-      if (qn > 0) {
-        soft_batch(0, qn);
-        qn = 0;
-      }
       ns = 0;
       if (last) break;
     }
+    if (qn > 0) soft_batch(0, qn);
     if (__any_sync(SFMM_FULL, tiny)) {
       if (lane == 0) f.fb[4 + atomicAdd(&f.fb[0], 1)] = item;
       __syncwarp();
