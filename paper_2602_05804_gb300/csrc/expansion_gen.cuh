@@ -594,6 +594,26 @@ static __device__ const signed char sfmm_l2l_table_0[4][4] = {
   {-1, -1, -1, 0}};
 static const int sfmm_moment_mi_0[1][3] = {{0,0,0}};
 
+template <typename T> __device__ __forceinline__ void sfmm_fold_0(const T* Q, T* q) {
+  q[0] = Q[0];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_m2l_fold_0(const T* D, const T* q, T* C) {
+  C[0] = fma(D[0], q[0], C[0]);
+  C[1] = fma(D[1], q[0], C[1]);
+  C[2] = fma(D[2], q[0], C[2]);
+  C[3] = fma(D[3], q[0], C[3]);
+}
+
+#define SFMM_NR_0 1  /* entries of a source row */
+#define SFMM_NS_0 4  /* sums of an interaction */
+#define SFMM_NX_0 1
+static __device__ const signed char sfmm_unfold_0[4][1][2] = {
+  {{0, 1}},
+  {{1, -1}},
+  {{2, -1}},
+  {{3, -1}}};
+
 template <typename T> __device__ __forceinline__ void sfmm_m2l_1(const T* D, const T* Q, T* C) {
   { T s = D[0] * Q[0];
     s = fma(D[1], Q[1], s);
@@ -718,6 +738,40 @@ static __device__ const signed char sfmm_l2l_table_1[13][13] = {
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, -1},
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0}};
 static const int sfmm_moment_mi_1[4][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}};
+
+template <typename T> __device__ __forceinline__ void sfmm_fold_1(const T* Q, T* q) {
+  q[0] = Q[0];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_m2l_fold_1(const T* D, const T* q, T* C) {
+  C[0] = fma(D[0], q[0], C[0]);
+  C[1] = fma(D[1], q[0], C[1]);
+  C[2] = fma(D[2], q[0], C[2]);
+  C[3] = fma(D[3], q[0], C[3]);
+  C[4] = fma(D[4], q[0], C[4]);
+  C[5] = fma(D[5], q[0], C[5]);
+  C[6] = fma(D[6], q[0], C[6]);
+  C[7] = fma(D[7], q[0], C[7]);
+  C[8] = fma(D[8], q[0], C[8]);
+}
+
+#define SFMM_NR_1 1  /* entries of a source row */
+#define SFMM_NS_1 9  /* sums of an interaction */
+#define SFMM_NX_1 2
+static __device__ const signed char sfmm_unfold_1[13][2][2] = {
+  {{0, 1}, {0, 0}},
+  {{1, -1}, {0, 0}},
+  {{2, -1}, {0, 0}},
+  {{3, -1}, {0, 0}},
+  {{1, -1}, {0, 0}},
+  {{2, -1}, {0, 0}},
+  {{3, -1}, {0, 0}},
+  {{4, 1}, {0, 0}},
+  {{5, 1}, {0, 0}},
+  {{6, 1}, {0, 0}},
+  {{7, 1}, {0, 0}},
+  {{8, 1}, {0, 0}},
+  {{4, -1}, {7, -1}}};
 
 template <typename T> __device__ __forceinline__ void sfmm_m2l_2(const T* D, const T* Q, T* C) {
   { T s = D[0] * Q[0];
@@ -1055,6 +1109,88 @@ static __device__ const signed char sfmm_l2l_table_2[29][29] = {
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, -1},
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0}};
 static const int sfmm_moment_mi_2[10][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}, {2,0,0}, {1,1,0}, {1,0,1}, {0,2,0}, {0,1,1}, {0,0,2}};
+
+template <typename T> __device__ __forceinline__ void sfmm_fold_2(const T* Q, T* q) {
+  q[0] = Q[0];
+  q[1] = Q[4] - Q[9];
+  q[2] = Q[5];
+  q[3] = Q[6];
+  q[4] = Q[7] - Q[9];
+  q[5] = Q[8];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_m2l_fold_2(const T* D, const T* q, T* C) {
+  { T s = D[4] * q[1];
+    s = fma(D[5], q[2], s);
+    s = fma(D[6], q[3], s);
+    s = fma(D[7], q[4], s);
+    s = fma(D[8], q[5], s);
+    C[0] += fma(D[0], q[0], s); }
+  C[1] = fma(D[1], q[0], C[1]);
+  C[2] = fma(D[2], q[0], C[2]);
+  C[3] = fma(D[3], q[0], C[3]);
+  C[4] = fma(D[4], q[0], C[4]);
+  C[5] = fma(D[5], q[0], C[5]);
+  C[6] = fma(D[6], q[0], C[6]);
+  C[7] = fma(D[7], q[0], C[7]);
+  C[8] = fma(D[8], q[0], C[8]);
+  C[9] = fma(D[10], q[1], C[9]);
+  C[9] = fma(D[11], q[2], C[9]);
+  C[9] = fma(D[12], q[3], C[9]);
+  C[9] = fma(D[13], q[4], C[9]);
+  C[9] = fma(D[14], q[5], C[9]);
+  C[10] = fma(D[11], q[1], C[10]);
+  C[10] = fma(D[13], q[2], C[10]);
+  C[10] = fma(D[14], q[3], C[10]);
+  C[10] = fma(D[16], q[4], C[10]);
+  C[10] = fma(D[17], q[5], C[10]);
+  C[11] = fma(D[12], q[1], C[11]);
+  C[11] = fma(D[14], q[2], C[11]);
+  C[11] = fma(D[15], q[3], C[11]);
+  C[11] = fma(D[17], q[4], C[11]);
+  C[11] = fma(D[18], q[5], C[11]);
+  C[12] = fma(D[10], q[0], C[12]);
+  C[13] = fma(D[11], q[0], C[13]);
+  C[14] = fma(D[12], q[0], C[14]);
+  C[15] = fma(D[13], q[0], C[15]);
+  C[16] = fma(D[14], q[0], C[16]);
+  C[17] = fma(D[16], q[0], C[17]);
+  C[18] = fma(D[17], q[0], C[18]);
+}
+
+#define SFMM_NR_2 6  /* entries of a source row */
+#define SFMM_NS_2 19  /* sums of an interaction */
+#define SFMM_NX_2 2
+static __device__ const signed char sfmm_unfold_2[29][2][2] = {
+  {{0, 1}, {0, 0}},
+  {{1, -1}, {0, 0}},
+  {{2, -1}, {0, 0}},
+  {{3, -1}, {0, 0}},
+  {{4, 1}, {0, 0}},
+  {{5, 1}, {0, 0}},
+  {{6, 1}, {0, 0}},
+  {{7, 1}, {0, 0}},
+  {{8, 1}, {0, 0}},
+  {{4, -1}, {7, -1}},
+  {{1, -1}, {9, -1}},
+  {{2, -1}, {10, -1}},
+  {{3, -1}, {11, -1}},
+  {{4, 1}, {0, 0}},
+  {{5, 1}, {0, 0}},
+  {{6, 1}, {0, 0}},
+  {{7, 1}, {0, 0}},
+  {{8, 1}, {0, 0}},
+  {{4, -1}, {7, -1}},
+  {{12, -1}, {0, 0}},
+  {{13, -1}, {0, 0}},
+  {{14, -1}, {0, 0}},
+  {{15, -1}, {0, 0}},
+  {{16, -1}, {0, 0}},
+  {{12, 1}, {15, 1}},
+  {{17, -1}, {0, 0}},
+  {{18, -1}, {0, 0}},
+  {{13, 1}, {17, 1}},
+  {{14, 1}, {18, 1}}};
 
 template <typename T> __device__ __forceinline__ void sfmm_m2l_3(const T* D, const T* Q, T* C) {
   { T s = D[0] * Q[0];
@@ -1869,6 +2005,182 @@ static __device__ const signed char sfmm_l2l_table_3[54][54] = {
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, -1},
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0}};
 static const int sfmm_moment_mi_3[20][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}, {2,0,0}, {1,1,0}, {1,0,1}, {0,2,0}, {0,1,1}, {0,0,2}, {3,0,0}, {2,1,0}, {2,0,1}, {1,2,0}, {1,1,1}, {1,0,2}, {0,3,0}, {0,2,1}, {0,1,2}, {0,0,3}};
+
+template <typename T> __device__ __forceinline__ void sfmm_fold_3(const T* Q, T* q) {
+  q[0] = Q[0];
+  q[1] = Q[4] - Q[9];
+  q[2] = Q[5];
+  q[3] = Q[6];
+  q[4] = Q[7] - Q[9];
+  q[5] = Q[8];
+  q[6] = Q[10] - Q[15];
+  q[7] = Q[11] - Q[18];
+  q[8] = Q[12] - Q[19];
+  q[9] = Q[13] - Q[15];
+  q[10] = Q[14];
+  q[11] = Q[16] - Q[18];
+  q[12] = Q[17] - Q[19];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_m2l_fold_3(const T* D, const T* q, T* C) {
+  { T s = D[4] * q[1];
+    s = fma(D[5], q[2], s);
+    s = fma(D[6], q[3], s);
+    s = fma(D[7], q[4], s);
+    s = fma(D[8], q[5], s);
+    s = fma(D[10], q[6], s);
+    s = fma(D[11], q[7], s);
+    s = fma(D[12], q[8], s);
+    s = fma(D[13], q[9], s);
+    s = fma(D[14], q[10], s);
+    s = fma(D[16], q[11], s);
+    s = fma(D[17], q[12], s);
+    C[0] += fma(D[0], q[0], s); }
+  { T s = D[10] * q[1];
+    s = fma(D[11], q[2], s);
+    s = fma(D[12], q[3], s);
+    s = fma(D[13], q[4], s);
+    s = fma(D[14], q[5], s);
+    C[1] += fma(D[1], q[0], s); }
+  { T s = D[11] * q[1];
+    s = fma(D[13], q[2], s);
+    s = fma(D[14], q[3], s);
+    s = fma(D[16], q[4], s);
+    s = fma(D[17], q[5], s);
+    C[2] += fma(D[2], q[0], s); }
+  { T s = D[12] * q[1];
+    s = fma(D[14], q[2], s);
+    s = fma(D[15], q[3], s);
+    s = fma(D[17], q[4], s);
+    s = fma(D[18], q[5], s);
+    C[3] += fma(D[3], q[0], s); }
+  C[4] = fma(D[4], q[0], C[4]);
+  C[5] = fma(D[5], q[0], C[5]);
+  C[6] = fma(D[6], q[0], C[6]);
+  C[7] = fma(D[7], q[0], C[7]);
+  C[8] = fma(D[8], q[0], C[8]);
+  C[9] = fma(D[10], q[0], C[9]);
+  C[10] = fma(D[11], q[0], C[10]);
+  C[11] = fma(D[12], q[0], C[11]);
+  C[12] = fma(D[13], q[0], C[12]);
+  C[13] = fma(D[14], q[0], C[13]);
+  C[14] = fma(D[16], q[0], C[14]);
+  C[15] = fma(D[17], q[0], C[15]);
+  C[16] = fma(D[20], q[6], C[16]);
+  C[16] = fma(D[21], q[7], C[16]);
+  C[16] = fma(D[22], q[8], C[16]);
+  C[16] = fma(D[23], q[9], C[16]);
+  C[16] = fma(D[24], q[10], C[16]);
+  C[16] = fma(D[26], q[11], C[16]);
+  C[16] = fma(D[27], q[12], C[16]);
+  C[17] = fma(D[21], q[6], C[17]);
+  C[17] = fma(D[23], q[7], C[17]);
+  C[17] = fma(D[24], q[8], C[17]);
+  C[17] = fma(D[26], q[9], C[17]);
+  C[17] = fma(D[27], q[10], C[17]);
+  C[17] = fma(D[30], q[11], C[17]);
+  C[17] = fma(D[31], q[12], C[17]);
+  C[18] = fma(D[22], q[6], C[18]);
+  C[18] = fma(D[24], q[7], C[18]);
+  C[18] = fma(D[25], q[8], C[18]);
+  C[18] = fma(D[27], q[9], C[18]);
+  C[18] = fma(D[28], q[10], C[18]);
+  C[18] = fma(D[31], q[11], C[18]);
+  C[18] = fma(D[32], q[12], C[18]);
+  C[19] = fma(D[20], q[1], C[19]);
+  C[19] = fma(D[21], q[2], C[19]);
+  C[19] = fma(D[22], q[3], C[19]);
+  C[19] = fma(D[23], q[4], C[19]);
+  C[19] = fma(D[24], q[5], C[19]);
+  C[20] = fma(D[21], q[1], C[20]);
+  C[20] = fma(D[23], q[2], C[20]);
+  C[20] = fma(D[24], q[3], C[20]);
+  C[20] = fma(D[26], q[4], C[20]);
+  C[20] = fma(D[27], q[5], C[20]);
+  C[21] = fma(D[22], q[1], C[21]);
+  C[21] = fma(D[24], q[2], C[21]);
+  C[21] = fma(D[25], q[3], C[21]);
+  C[21] = fma(D[27], q[4], C[21]);
+  C[21] = fma(D[28], q[5], C[21]);
+  C[22] = fma(D[23], q[1], C[22]);
+  C[22] = fma(D[26], q[2], C[22]);
+  C[22] = fma(D[27], q[3], C[22]);
+  C[22] = fma(D[30], q[4], C[22]);
+  C[22] = fma(D[31], q[5], C[22]);
+  C[23] = fma(D[24], q[1], C[23]);
+  C[23] = fma(D[27], q[2], C[23]);
+  C[23] = fma(D[28], q[3], C[23]);
+  C[23] = fma(D[31], q[4], C[23]);
+  C[23] = fma(D[32], q[5], C[23]);
+  C[24] = fma(D[20], q[0], C[24]);
+  C[25] = fma(D[21], q[0], C[25]);
+  C[26] = fma(D[22], q[0], C[26]);
+  C[27] = fma(D[23], q[0], C[27]);
+  C[28] = fma(D[24], q[0], C[28]);
+  C[29] = fma(D[26], q[0], C[29]);
+  C[30] = fma(D[27], q[0], C[30]);
+  C[31] = fma(D[30], q[0], C[31]);
+  C[32] = fma(D[31], q[0], C[32]);
+}
+
+#define SFMM_NR_3 13  /* entries of a source row */
+#define SFMM_NS_3 33  /* sums of an interaction */
+#define SFMM_NX_3 4
+static __device__ const signed char sfmm_unfold_3[54][4][2] = {
+  {{0, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{1, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{2, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{3, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{4, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{5, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{6, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{7, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{8, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{4, -1}, {7, -1}, {0, 0}, {0, 0}},
+  {{9, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{10, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{11, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{12, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{13, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{9, 1}, {12, 1}, {0, 0}, {0, 0}},
+  {{14, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{15, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{10, 1}, {14, 1}, {0, 0}, {0, 0}},
+  {{11, 1}, {15, 1}, {0, 0}, {0, 0}},
+  {{1, -1}, {16, -1}, {0, 0}, {0, 0}},
+  {{2, -1}, {17, -1}, {0, 0}, {0, 0}},
+  {{3, -1}, {18, -1}, {0, 0}, {0, 0}},
+  {{4, 1}, {19, 1}, {0, 0}, {0, 0}},
+  {{5, 1}, {20, 1}, {0, 0}, {0, 0}},
+  {{6, 1}, {21, 1}, {0, 0}, {0, 0}},
+  {{7, 1}, {22, 1}, {0, 0}, {0, 0}},
+  {{8, 1}, {23, 1}, {0, 0}, {0, 0}},
+  {{4, -1}, {19, -1}, {7, -1}, {22, -1}},
+  {{9, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{10, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{11, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{12, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{13, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{9, 1}, {12, 1}, {0, 0}, {0, 0}},
+  {{14, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{15, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{10, 1}, {14, 1}, {0, 0}, {0, 0}},
+  {{11, 1}, {15, 1}, {0, 0}, {0, 0}},
+  {{24, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{25, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{26, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{27, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{28, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{24, -1}, {27, -1}, {0, 0}, {0, 0}},
+  {{29, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{30, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{25, -1}, {29, -1}, {0, 0}, {0, 0}},
+  {{26, -1}, {30, -1}, {0, 0}, {0, 0}},
+  {{31, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{32, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{27, -1}, {31, -1}, {0, 0}, {0, 0}},
+  {{28, -1}, {32, -1}, {0, 0}, {0, 0}},
+  {{24, 1}, {27, 2}, {31, 1}, {0, 0}}};
 
 template <typename T> __device__ __forceinline__ void sfmm_m2l_4(const T* D, const T* Q, T* C) {
   { T s = D[0] * Q[0];
@@ -3646,4 +3958,916 @@ static __device__ const signed char sfmm_l2l_table_4[90][90] = {
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, -1},
   {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0}};
 static const int sfmm_moment_mi_4[35][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}, {2,0,0}, {1,1,0}, {1,0,1}, {0,2,0}, {0,1,1}, {0,0,2}, {3,0,0}, {2,1,0}, {2,0,1}, {1,2,0}, {1,1,1}, {1,0,2}, {0,3,0}, {0,2,1}, {0,1,2}, {0,0,3}, {4,0,0}, {3,1,0}, {3,0,1}, {2,2,0}, {2,1,1}, {2,0,2}, {1,3,0}, {1,2,1}, {1,1,2}, {1,0,3}, {0,4,0}, {0,3,1}, {0,2,2}, {0,1,3}, {0,0,4}};
+
+template <typename T> __device__ __forceinline__ void sfmm_fold_4(const T* Q, T* q) {
+  q[0] = Q[0];
+  q[1] = Q[4] - Q[9];
+  q[2] = Q[5];
+  q[3] = Q[6];
+  q[4] = Q[7] - Q[9];
+  q[5] = Q[8];
+  q[6] = Q[10] - Q[15];
+  q[7] = Q[11] - Q[18];
+  q[8] = Q[12] - Q[19];
+  q[9] = Q[13] - Q[15];
+  q[10] = Q[14];
+  q[11] = Q[16] - Q[18];
+  q[12] = Q[17] - Q[19];
+  q[13] = Q[20] - Q[25] + Q[34];
+  q[14] = Q[21] - Q[28];
+  q[15] = Q[22] - Q[29];
+  q[16] = Q[23] - Q[25] - Q[32] + T(2.0) * Q[34];
+  q[17] = Q[24] - Q[33];
+  q[18] = Q[26] - Q[28];
+  q[19] = Q[27] - Q[29];
+  q[20] = Q[30] - Q[32] + Q[34];
+  q[21] = Q[31] - Q[33];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_m2l_fold_4(const T* D, const T* q, T* C) {
+  { T s = D[4] * q[1];
+    s = fma(D[5], q[2], s);
+    s = fma(D[6], q[3], s);
+    s = fma(D[7], q[4], s);
+    s = fma(D[8], q[5], s);
+    s = fma(D[10], q[6], s);
+    s = fma(D[11], q[7], s);
+    s = fma(D[12], q[8], s);
+    s = fma(D[13], q[9], s);
+    s = fma(D[14], q[10], s);
+    s = fma(D[16], q[11], s);
+    s = fma(D[17], q[12], s);
+    s = fma(D[20], q[13], s);
+    s = fma(D[21], q[14], s);
+    s = fma(D[22], q[15], s);
+    s = fma(D[23], q[16], s);
+    s = fma(D[24], q[17], s);
+    s = fma(D[26], q[18], s);
+    s = fma(D[27], q[19], s);
+    s = fma(D[30], q[20], s);
+    s = fma(D[31], q[21], s);
+    C[0] += fma(D[0], q[0], s); }
+  { T s = D[10] * q[1];
+    s = fma(D[11], q[2], s);
+    s = fma(D[12], q[3], s);
+    s = fma(D[13], q[4], s);
+    s = fma(D[14], q[5], s);
+    s = fma(D[20], q[6], s);
+    s = fma(D[21], q[7], s);
+    s = fma(D[22], q[8], s);
+    s = fma(D[23], q[9], s);
+    s = fma(D[24], q[10], s);
+    s = fma(D[26], q[11], s);
+    s = fma(D[27], q[12], s);
+    C[1] += fma(D[1], q[0], s); }
+  { T s = D[11] * q[1];
+    s = fma(D[13], q[2], s);
+    s = fma(D[14], q[3], s);
+    s = fma(D[16], q[4], s);
+    s = fma(D[17], q[5], s);
+    s = fma(D[21], q[6], s);
+    s = fma(D[23], q[7], s);
+    s = fma(D[24], q[8], s);
+    s = fma(D[26], q[9], s);
+    s = fma(D[27], q[10], s);
+    s = fma(D[30], q[11], s);
+    s = fma(D[31], q[12], s);
+    C[2] += fma(D[2], q[0], s); }
+  { T s = D[12] * q[1];
+    s = fma(D[14], q[2], s);
+    s = fma(D[15], q[3], s);
+    s = fma(D[17], q[4], s);
+    s = fma(D[18], q[5], s);
+    s = fma(D[22], q[6], s);
+    s = fma(D[24], q[7], s);
+    s = fma(D[25], q[8], s);
+    s = fma(D[27], q[9], s);
+    s = fma(D[28], q[10], s);
+    s = fma(D[31], q[11], s);
+    s = fma(D[32], q[12], s);
+    C[3] += fma(D[3], q[0], s); }
+  { T s = D[20] * q[1];
+    s = fma(D[21], q[2], s);
+    s = fma(D[22], q[3], s);
+    s = fma(D[23], q[4], s);
+    s = fma(D[24], q[5], s);
+    C[4] += fma(D[4], q[0], s); }
+  { T s = D[21] * q[1];
+    s = fma(D[23], q[2], s);
+    s = fma(D[24], q[3], s);
+    s = fma(D[26], q[4], s);
+    s = fma(D[27], q[5], s);
+    C[5] += fma(D[5], q[0], s); }
+  { T s = D[22] * q[1];
+    s = fma(D[24], q[2], s);
+    s = fma(D[25], q[3], s);
+    s = fma(D[27], q[4], s);
+    s = fma(D[28], q[5], s);
+    C[6] += fma(D[6], q[0], s); }
+  { T s = D[23] * q[1];
+    s = fma(D[26], q[2], s);
+    s = fma(D[27], q[3], s);
+    s = fma(D[30], q[4], s);
+    s = fma(D[31], q[5], s);
+    C[7] += fma(D[7], q[0], s); }
+  { T s = D[24] * q[1];
+    s = fma(D[27], q[2], s);
+    s = fma(D[28], q[3], s);
+    s = fma(D[31], q[4], s);
+    s = fma(D[32], q[5], s);
+    C[8] += fma(D[8], q[0], s); }
+  C[9] = fma(D[10], q[0], C[9]);
+  C[10] = fma(D[11], q[0], C[10]);
+  C[11] = fma(D[12], q[0], C[11]);
+  C[12] = fma(D[13], q[0], C[12]);
+  C[13] = fma(D[14], q[0], C[13]);
+  C[14] = fma(D[16], q[0], C[14]);
+  C[15] = fma(D[17], q[0], C[15]);
+  C[16] = fma(D[20], q[0], C[16]);
+  C[17] = fma(D[21], q[0], C[17]);
+  C[18] = fma(D[22], q[0], C[18]);
+  C[19] = fma(D[23], q[0], C[19]);
+  C[20] = fma(D[24], q[0], C[20]);
+  C[21] = fma(D[26], q[0], C[21]);
+  C[22] = fma(D[27], q[0], C[22]);
+  C[23] = fma(D[30], q[0], C[23]);
+  C[24] = fma(D[31], q[0], C[24]);
+  C[25] = fma(D[35], q[13], C[25]);
+  C[25] = fma(D[36], q[14], C[25]);
+  C[25] = fma(D[37], q[15], C[25]);
+  C[25] = fma(D[38], q[16], C[25]);
+  C[25] = fma(D[39], q[17], C[25]);
+  C[25] = fma(D[41], q[18], C[25]);
+  C[25] = fma(D[42], q[19], C[25]);
+  C[25] = fma(D[45], q[20], C[25]);
+  C[25] = fma(D[46], q[21], C[25]);
+  C[26] = fma(D[36], q[13], C[26]);
+  C[26] = fma(D[38], q[14], C[26]);
+  C[26] = fma(D[39], q[15], C[26]);
+  C[26] = fma(D[41], q[16], C[26]);
+  C[26] = fma(D[42], q[17], C[26]);
+  C[26] = fma(D[45], q[18], C[26]);
+  C[26] = fma(D[46], q[19], C[26]);
+  C[26] = fma(D[50], q[20], C[26]);
+  C[26] = fma(D[51], q[21], C[26]);
+  C[27] = fma(D[37], q[13], C[27]);
+  C[27] = fma(D[39], q[14], C[27]);
+  C[27] = fma(D[40], q[15], C[27]);
+  C[27] = fma(D[42], q[16], C[27]);
+  C[27] = fma(D[43], q[17], C[27]);
+  C[27] = fma(D[46], q[18], C[27]);
+  C[27] = fma(D[47], q[19], C[27]);
+  C[27] = fma(D[51], q[20], C[27]);
+  C[27] = fma(D[52], q[21], C[27]);
+  C[28] = fma(D[35], q[6], C[28]);
+  C[28] = fma(D[36], q[7], C[28]);
+  C[28] = fma(D[37], q[8], C[28]);
+  C[28] = fma(D[38], q[9], C[28]);
+  C[28] = fma(D[39], q[10], C[28]);
+  C[28] = fma(D[41], q[11], C[28]);
+  C[28] = fma(D[42], q[12], C[28]);
+  C[29] = fma(D[36], q[6], C[29]);
+  C[29] = fma(D[38], q[7], C[29]);
+  C[29] = fma(D[39], q[8], C[29]);
+  C[29] = fma(D[41], q[9], C[29]);
+  C[29] = fma(D[42], q[10], C[29]);
+  C[29] = fma(D[45], q[11], C[29]);
+  C[29] = fma(D[46], q[12], C[29]);
+  C[30] = fma(D[37], q[6], C[30]);
+  C[30] = fma(D[39], q[7], C[30]);
+  C[30] = fma(D[40], q[8], C[30]);
+  C[30] = fma(D[42], q[9], C[30]);
+  C[30] = fma(D[43], q[10], C[30]);
+  C[30] = fma(D[46], q[11], C[30]);
+  C[30] = fma(D[47], q[12], C[30]);
+  C[31] = fma(D[38], q[6], C[31]);
+  C[31] = fma(D[41], q[7], C[31]);
+  C[31] = fma(D[42], q[8], C[31]);
+  C[31] = fma(D[45], q[9], C[31]);
+  C[31] = fma(D[46], q[10], C[31]);
+  C[31] = fma(D[50], q[11], C[31]);
+  C[31] = fma(D[51], q[12], C[31]);
+  C[32] = fma(D[39], q[6], C[32]);
+  C[32] = fma(D[42], q[7], C[32]);
+  C[32] = fma(D[43], q[8], C[32]);
+  C[32] = fma(D[46], q[9], C[32]);
+  C[32] = fma(D[47], q[10], C[32]);
+  C[32] = fma(D[51], q[11], C[32]);
+  C[32] = fma(D[52], q[12], C[32]);
+  C[33] = fma(D[35], q[1], C[33]);
+  C[33] = fma(D[36], q[2], C[33]);
+  C[33] = fma(D[37], q[3], C[33]);
+  C[33] = fma(D[38], q[4], C[33]);
+  C[33] = fma(D[39], q[5], C[33]);
+  C[34] = fma(D[36], q[1], C[34]);
+  C[34] = fma(D[38], q[2], C[34]);
+  C[34] = fma(D[39], q[3], C[34]);
+  C[34] = fma(D[41], q[4], C[34]);
+  C[34] = fma(D[42], q[5], C[34]);
+  C[35] = fma(D[37], q[1], C[35]);
+  C[35] = fma(D[39], q[2], C[35]);
+  C[35] = fma(D[40], q[3], C[35]);
+  C[35] = fma(D[42], q[4], C[35]);
+  C[35] = fma(D[43], q[5], C[35]);
+  C[36] = fma(D[38], q[1], C[36]);
+  C[36] = fma(D[41], q[2], C[36]);
+  C[36] = fma(D[42], q[3], C[36]);
+  C[36] = fma(D[45], q[4], C[36]);
+  C[36] = fma(D[46], q[5], C[36]);
+  C[37] = fma(D[39], q[1], C[37]);
+  C[37] = fma(D[42], q[2], C[37]);
+  C[37] = fma(D[43], q[3], C[37]);
+  C[37] = fma(D[46], q[4], C[37]);
+  C[37] = fma(D[47], q[5], C[37]);
+  C[38] = fma(D[41], q[1], C[38]);
+  C[38] = fma(D[45], q[2], C[38]);
+  C[38] = fma(D[46], q[3], C[38]);
+  C[38] = fma(D[50], q[4], C[38]);
+  C[38] = fma(D[51], q[5], C[38]);
+  C[39] = fma(D[42], q[1], C[39]);
+  C[39] = fma(D[46], q[2], C[39]);
+  C[39] = fma(D[47], q[3], C[39]);
+  C[39] = fma(D[51], q[4], C[39]);
+  C[39] = fma(D[52], q[5], C[39]);
+  C[40] = fma(D[35], q[0], C[40]);
+  C[41] = fma(D[36], q[0], C[41]);
+  C[42] = fma(D[37], q[0], C[42]);
+  C[43] = fma(D[38], q[0], C[43]);
+  C[44] = fma(D[39], q[0], C[44]);
+  C[45] = fma(D[41], q[0], C[45]);
+  C[46] = fma(D[42], q[0], C[46]);
+  C[47] = fma(D[45], q[0], C[47]);
+  C[48] = fma(D[46], q[0], C[48]);
+  C[49] = fma(D[50], q[0], C[49]);
+  C[50] = fma(D[51], q[0], C[50]);
+}
+
+#define SFMM_NR_4 22  /* entries of a source row */
+#define SFMM_NS_4 51  /* sums of an interaction */
+#define SFMM_NX_4 4
+static __device__ const signed char sfmm_unfold_4[90][4][2] = {
+  {{0, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{1, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{2, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{3, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{4, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{5, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{6, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{7, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{8, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{4, -1}, {7, -1}, {0, 0}, {0, 0}},
+  {{9, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{10, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{11, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{12, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{13, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{9, 1}, {12, 1}, {0, 0}, {0, 0}},
+  {{14, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{15, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{10, 1}, {14, 1}, {0, 0}, {0, 0}},
+  {{11, 1}, {15, 1}, {0, 0}, {0, 0}},
+  {{16, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{17, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{18, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{19, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{20, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{16, -1}, {19, -1}, {0, 0}, {0, 0}},
+  {{21, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{22, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{17, -1}, {21, -1}, {0, 0}, {0, 0}},
+  {{18, -1}, {22, -1}, {0, 0}, {0, 0}},
+  {{23, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{24, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{19, -1}, {23, -1}, {0, 0}, {0, 0}},
+  {{20, -1}, {24, -1}, {0, 0}, {0, 0}},
+  {{16, 1}, {19, 2}, {23, 1}, {0, 0}},
+  {{1, -1}, {25, -1}, {0, 0}, {0, 0}},
+  {{2, -1}, {26, -1}, {0, 0}, {0, 0}},
+  {{3, -1}, {27, -1}, {0, 0}, {0, 0}},
+  {{4, 1}, {28, 1}, {0, 0}, {0, 0}},
+  {{5, 1}, {29, 1}, {0, 0}, {0, 0}},
+  {{6, 1}, {30, 1}, {0, 0}, {0, 0}},
+  {{7, 1}, {31, 1}, {0, 0}, {0, 0}},
+  {{8, 1}, {32, 1}, {0, 0}, {0, 0}},
+  {{4, -1}, {28, -1}, {7, -1}, {31, -1}},
+  {{9, -1}, {33, -1}, {0, 0}, {0, 0}},
+  {{10, -1}, {34, -1}, {0, 0}, {0, 0}},
+  {{11, -1}, {35, -1}, {0, 0}, {0, 0}},
+  {{12, -1}, {36, -1}, {0, 0}, {0, 0}},
+  {{13, -1}, {37, -1}, {0, 0}, {0, 0}},
+  {{9, 1}, {33, 1}, {12, 1}, {36, 1}},
+  {{14, -1}, {38, -1}, {0, 0}, {0, 0}},
+  {{15, -1}, {39, -1}, {0, 0}, {0, 0}},
+  {{10, 1}, {34, 1}, {14, 1}, {38, 1}},
+  {{11, 1}, {35, 1}, {15, 1}, {39, 1}},
+  {{16, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{17, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{18, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{19, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{20, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{16, -1}, {19, -1}, {0, 0}, {0, 0}},
+  {{21, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{22, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{17, -1}, {21, -1}, {0, 0}, {0, 0}},
+  {{18, -1}, {22, -1}, {0, 0}, {0, 0}},
+  {{23, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{24, 1}, {0, 0}, {0, 0}, {0, 0}},
+  {{19, -1}, {23, -1}, {0, 0}, {0, 0}},
+  {{20, -1}, {24, -1}, {0, 0}, {0, 0}},
+  {{16, 1}, {19, 2}, {23, 1}, {0, 0}},
+  {{40, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{41, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{42, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{43, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{44, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{40, 1}, {43, 1}, {0, 0}, {0, 0}},
+  {{45, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{46, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{41, 1}, {45, 1}, {0, 0}, {0, 0}},
+  {{42, 1}, {46, 1}, {0, 0}, {0, 0}},
+  {{47, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{48, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{43, 1}, {47, 1}, {0, 0}, {0, 0}},
+  {{44, 1}, {48, 1}, {0, 0}, {0, 0}},
+  {{40, -1}, {43, -2}, {47, -1}, {0, 0}},
+  {{49, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{50, -1}, {0, 0}, {0, 0}, {0, 0}},
+  {{45, 1}, {49, 1}, {0, 0}, {0, 0}},
+  {{46, 1}, {50, 1}, {0, 0}, {0, 0}},
+  {{41, -1}, {45, -2}, {49, -1}, {0, 0}},
+  {{42, -1}, {46, -2}, {50, -1}, {0, 0}}};
+
+template <typename T> __device__ __forceinline__ void sfmm_derivs_fold_1(T x, T y, T z, T rinv, T* D) {
+  const T ri2 = rinv * rinv, b0 = rinv;
+  const T b1 = b0 * (ri2 * T(-1.0));
+  const T R0_100 = x * b1;
+  const T R0_010 = y * b1;
+  const T R0_001 = z * b1;
+  D[0] = b0;
+  D[1] = R0_100;
+  D[2] = R0_010;
+  D[3] = R0_001;
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_uderivs_fold_1(T x, T y, T z, T rinv, T* D) {
+  const T R0_100 = x * T(-1.0);
+  const T R0_010 = y * T(-1.0);
+  const T R0_001 = z * T(-1.0);
+  T s = rinv;
+  D[0] = T(1.0) * s;
+  s = s * rinv;
+  D[1] = R0_100 * s;
+  D[2] = R0_010 * s;
+  D[3] = R0_001 * s;
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_derivs_fold_2(T x, T y, T z, T rinv, T* D) {
+  const T ri2 = rinv * rinv, b0 = rinv;
+  const T b1 = b0 * (ri2 * T(-1.0));
+  const T b2 = b1 * (ri2 * T(-3.0));
+  const T R0_100 = x * b1;
+  const T R0_010 = y * b1;
+  const T R0_001 = z * b1;
+  const T R1_100 = x * b2;
+  const T R0_200 = fma(x, R1_100, b1);
+  const T R1_010 = y * b2;
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * b2;
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, b1);
+  const T R0_011 = y * R1_001;
+  D[0] = b0;
+  D[1] = R0_100;
+  D[2] = R0_010;
+  D[3] = R0_001;
+  D[4] = R0_200;
+  D[5] = R0_110;
+  D[6] = R0_101;
+  D[7] = R0_020;
+  D[8] = R0_011;
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_uderivs_fold_2(T x, T y, T z, T rinv, T* D) {
+  const T R0_100 = x * T(-1.0);
+  const T R0_010 = y * T(-1.0);
+  const T R0_001 = z * T(-1.0);
+  const T R1_100 = x * T(3.0);
+  const T R0_200 = fma(x, R1_100, T(-1.0));
+  const T R1_010 = y * T(3.0);
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * T(3.0);
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, T(-1.0));
+  const T R0_011 = y * R1_001;
+  T s = rinv;
+  D[0] = T(1.0) * s;
+  s = s * rinv;
+  D[1] = R0_100 * s;
+  D[2] = R0_010 * s;
+  D[3] = R0_001 * s;
+  s = s * rinv;
+  D[4] = R0_200 * s;
+  D[5] = R0_110 * s;
+  D[6] = R0_101 * s;
+  D[7] = R0_020 * s;
+  D[8] = R0_011 * s;
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_derivs_fold_3(T x, T y, T z, T rinv, T* D) {
+  const T ri2 = rinv * rinv, b0 = rinv;
+  const T b1 = b0 * (ri2 * T(-1.0));
+  const T b2 = b1 * (ri2 * T(-3.0));
+  const T b3 = b2 * (ri2 * T(-5.0));
+  const T R0_100 = x * b1;
+  const T R0_010 = y * b1;
+  const T R0_001 = z * b1;
+  const T R1_100 = x * b2;
+  const T R0_200 = fma(x, R1_100, b1);
+  const T R1_010 = y * b2;
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * b2;
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, b1);
+  const T R0_011 = y * R1_001;
+  const T R2_100 = x * b3;
+  const T R1_200 = fma(x, R2_100, b2);
+  const T R0_300 = fma(x, R1_200, T(2.0) * R1_100);
+  const T R0_210 = y * R1_200;
+  const T R0_201 = z * R1_200;
+  const T R2_010 = y * b3;
+  const T R1_020 = fma(y, R2_010, b2);
+  const T R0_120 = x * R1_020;
+  const T R2_001 = z * b3;
+  const T R1_011 = y * R2_001;
+  const T R0_111 = x * R1_011;
+  const T R0_030 = fma(y, R1_020, T(2.0) * R1_010);
+  const T R0_021 = z * R1_020;
+  D[0] = b0;
+  D[1] = R0_100;
+  D[2] = R0_010;
+  D[3] = R0_001;
+  D[4] = R0_200;
+  D[5] = R0_110;
+  D[6] = R0_101;
+  D[7] = R0_020;
+  D[8] = R0_011;
+  D[10] = R0_300;
+  D[11] = R0_210;
+  D[12] = R0_201;
+  D[13] = R0_120;
+  D[14] = R0_111;
+  D[16] = R0_030;
+  D[17] = R0_021;
+  D[15] = -D[10] - D[13];
+  D[18] = -D[11] - D[16];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_uderivs_fold_3(T x, T y, T z, T rinv, T* D) {
+  const T R0_100 = x * T(-1.0);
+  const T R0_010 = y * T(-1.0);
+  const T R0_001 = z * T(-1.0);
+  const T R1_100 = x * T(3.0);
+  const T R0_200 = fma(x, R1_100, T(-1.0));
+  const T R1_010 = y * T(3.0);
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * T(3.0);
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, T(-1.0));
+  const T R0_011 = y * R1_001;
+  const T R2_100 = x * T(-15.0);
+  const T R1_200 = fma(x, R2_100, T(3.0));
+  const T R0_300 = fma(x, R1_200, T(2.0) * R1_100);
+  const T R0_210 = y * R1_200;
+  const T R0_201 = z * R1_200;
+  const T R2_010 = y * T(-15.0);
+  const T R1_020 = fma(y, R2_010, T(3.0));
+  const T R0_120 = x * R1_020;
+  const T R2_001 = z * T(-15.0);
+  const T R1_011 = y * R2_001;
+  const T R0_111 = x * R1_011;
+  const T R0_030 = fma(y, R1_020, T(2.0) * R1_010);
+  const T R0_021 = z * R1_020;
+  T s = rinv;
+  D[0] = T(1.0) * s;
+  s = s * rinv;
+  D[1] = R0_100 * s;
+  D[2] = R0_010 * s;
+  D[3] = R0_001 * s;
+  s = s * rinv;
+  D[4] = R0_200 * s;
+  D[5] = R0_110 * s;
+  D[6] = R0_101 * s;
+  D[7] = R0_020 * s;
+  D[8] = R0_011 * s;
+  s = s * rinv;
+  D[10] = R0_300 * s;
+  D[11] = R0_210 * s;
+  D[12] = R0_201 * s;
+  D[13] = R0_120 * s;
+  D[14] = R0_111 * s;
+  D[16] = R0_030 * s;
+  D[17] = R0_021 * s;
+  D[15] = -D[10] - D[13];
+  D[18] = -D[11] - D[16];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_derivs_fold_4(T x, T y, T z, T rinv, T* D) {
+  const T ri2 = rinv * rinv, b0 = rinv;
+  const T b1 = b0 * (ri2 * T(-1.0));
+  const T b2 = b1 * (ri2 * T(-3.0));
+  const T b3 = b2 * (ri2 * T(-5.0));
+  const T b4 = b3 * (ri2 * T(-7.0));
+  const T R0_100 = x * b1;
+  const T R0_010 = y * b1;
+  const T R0_001 = z * b1;
+  const T R1_100 = x * b2;
+  const T R0_200 = fma(x, R1_100, b1);
+  const T R1_010 = y * b2;
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * b2;
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, b1);
+  const T R0_011 = y * R1_001;
+  const T R2_100 = x * b3;
+  const T R1_200 = fma(x, R2_100, b2);
+  const T R0_300 = fma(x, R1_200, T(2.0) * R1_100);
+  const T R0_210 = y * R1_200;
+  const T R0_201 = z * R1_200;
+  const T R2_010 = y * b3;
+  const T R1_020 = fma(y, R2_010, b2);
+  const T R0_120 = x * R1_020;
+  const T R2_001 = z * b3;
+  const T R1_011 = y * R2_001;
+  const T R0_111 = x * R1_011;
+  const T R0_030 = fma(y, R1_020, T(2.0) * R1_010);
+  const T R0_021 = z * R1_020;
+  const T R3_100 = x * b4;
+  const T R2_200 = fma(x, R3_100, b3);
+  const T R1_300 = fma(x, R2_200, T(2.0) * R2_100);
+  const T R0_400 = fma(x, R1_300, T(3.0) * R1_200);
+  const T R0_310 = y * R1_300;
+  const T R0_301 = z * R1_300;
+  const T R3_010 = y * b4;
+  const T R2_020 = fma(y, R3_010, b3);
+  const T R1_120 = x * R2_020;
+  const T R0_220 = fma(x, R1_120, R1_020);
+  const T R1_201 = z * R2_200;
+  const T R0_211 = y * R1_201;
+  const T R1_030 = fma(y, R2_020, T(2.0) * R2_010);
+  const T R0_130 = x * R1_030;
+  const T R1_021 = z * R2_020;
+  const T R0_121 = x * R1_021;
+  const T R0_040 = fma(y, R1_030, T(3.0) * R1_020);
+  const T R0_031 = z * R1_030;
+  D[0] = b0;
+  D[1] = R0_100;
+  D[2] = R0_010;
+  D[3] = R0_001;
+  D[4] = R0_200;
+  D[5] = R0_110;
+  D[6] = R0_101;
+  D[7] = R0_020;
+  D[8] = R0_011;
+  D[10] = R0_300;
+  D[11] = R0_210;
+  D[12] = R0_201;
+  D[13] = R0_120;
+  D[14] = R0_111;
+  D[16] = R0_030;
+  D[17] = R0_021;
+  D[15] = -D[10] - D[13];
+  D[18] = -D[11] - D[16];
+  D[20] = R0_400;
+  D[21] = R0_310;
+  D[22] = R0_301;
+  D[23] = R0_220;
+  D[24] = R0_211;
+  D[26] = R0_130;
+  D[27] = R0_121;
+  D[30] = R0_040;
+  D[31] = R0_031;
+  D[25] = -D[20] - D[23];
+  D[28] = -D[21] - D[26];
+  D[32] = -D[23] - D[30];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_uderivs_fold_4(T x, T y, T z, T rinv, T* D) {
+  const T R0_100 = x * T(-1.0);
+  const T R0_010 = y * T(-1.0);
+  const T R0_001 = z * T(-1.0);
+  const T R1_100 = x * T(3.0);
+  const T R0_200 = fma(x, R1_100, T(-1.0));
+  const T R1_010 = y * T(3.0);
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * T(3.0);
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, T(-1.0));
+  const T R0_011 = y * R1_001;
+  const T R2_100 = x * T(-15.0);
+  const T R1_200 = fma(x, R2_100, T(3.0));
+  const T R0_300 = fma(x, R1_200, T(2.0) * R1_100);
+  const T R0_210 = y * R1_200;
+  const T R0_201 = z * R1_200;
+  const T R2_010 = y * T(-15.0);
+  const T R1_020 = fma(y, R2_010, T(3.0));
+  const T R0_120 = x * R1_020;
+  const T R2_001 = z * T(-15.0);
+  const T R1_011 = y * R2_001;
+  const T R0_111 = x * R1_011;
+  const T R0_030 = fma(y, R1_020, T(2.0) * R1_010);
+  const T R0_021 = z * R1_020;
+  const T R3_100 = x * T(105.0);
+  const T R2_200 = fma(x, R3_100, T(-15.0));
+  const T R1_300 = fma(x, R2_200, T(2.0) * R2_100);
+  const T R0_400 = fma(x, R1_300, T(3.0) * R1_200);
+  const T R0_310 = y * R1_300;
+  const T R0_301 = z * R1_300;
+  const T R3_010 = y * T(105.0);
+  const T R2_020 = fma(y, R3_010, T(-15.0));
+  const T R1_120 = x * R2_020;
+  const T R0_220 = fma(x, R1_120, R1_020);
+  const T R1_201 = z * R2_200;
+  const T R0_211 = y * R1_201;
+  const T R1_030 = fma(y, R2_020, T(2.0) * R2_010);
+  const T R0_130 = x * R1_030;
+  const T R1_021 = z * R2_020;
+  const T R0_121 = x * R1_021;
+  const T R0_040 = fma(y, R1_030, T(3.0) * R1_020);
+  const T R0_031 = z * R1_030;
+  T s = rinv;
+  D[0] = T(1.0) * s;
+  s = s * rinv;
+  D[1] = R0_100 * s;
+  D[2] = R0_010 * s;
+  D[3] = R0_001 * s;
+  s = s * rinv;
+  D[4] = R0_200 * s;
+  D[5] = R0_110 * s;
+  D[6] = R0_101 * s;
+  D[7] = R0_020 * s;
+  D[8] = R0_011 * s;
+  s = s * rinv;
+  D[10] = R0_300 * s;
+  D[11] = R0_210 * s;
+  D[12] = R0_201 * s;
+  D[13] = R0_120 * s;
+  D[14] = R0_111 * s;
+  D[16] = R0_030 * s;
+  D[17] = R0_021 * s;
+  D[15] = -D[10] - D[13];
+  D[18] = -D[11] - D[16];
+  s = s * rinv;
+  D[20] = R0_400 * s;
+  D[21] = R0_310 * s;
+  D[22] = R0_301 * s;
+  D[23] = R0_220 * s;
+  D[24] = R0_211 * s;
+  D[26] = R0_130 * s;
+  D[27] = R0_121 * s;
+  D[30] = R0_040 * s;
+  D[31] = R0_031 * s;
+  D[25] = -D[20] - D[23];
+  D[28] = -D[21] - D[26];
+  D[32] = -D[23] - D[30];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_derivs_fold_5(T x, T y, T z, T rinv, T* D) {
+  const T ri2 = rinv * rinv, b0 = rinv;
+  const T b1 = b0 * (ri2 * T(-1.0));
+  const T b2 = b1 * (ri2 * T(-3.0));
+  const T b3 = b2 * (ri2 * T(-5.0));
+  const T b4 = b3 * (ri2 * T(-7.0));
+  const T b5 = b4 * (ri2 * T(-9.0));
+  const T R0_100 = x * b1;
+  const T R0_010 = y * b1;
+  const T R0_001 = z * b1;
+  const T R1_100 = x * b2;
+  const T R0_200 = fma(x, R1_100, b1);
+  const T R1_010 = y * b2;
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * b2;
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, b1);
+  const T R0_011 = y * R1_001;
+  const T R2_100 = x * b3;
+  const T R1_200 = fma(x, R2_100, b2);
+  const T R0_300 = fma(x, R1_200, T(2.0) * R1_100);
+  const T R0_210 = y * R1_200;
+  const T R0_201 = z * R1_200;
+  const T R2_010 = y * b3;
+  const T R1_020 = fma(y, R2_010, b2);
+  const T R0_120 = x * R1_020;
+  const T R2_001 = z * b3;
+  const T R1_011 = y * R2_001;
+  const T R0_111 = x * R1_011;
+  const T R0_030 = fma(y, R1_020, T(2.0) * R1_010);
+  const T R0_021 = z * R1_020;
+  const T R3_100 = x * b4;
+  const T R2_200 = fma(x, R3_100, b3);
+  const T R1_300 = fma(x, R2_200, T(2.0) * R2_100);
+  const T R0_400 = fma(x, R1_300, T(3.0) * R1_200);
+  const T R0_310 = y * R1_300;
+  const T R0_301 = z * R1_300;
+  const T R3_010 = y * b4;
+  const T R2_020 = fma(y, R3_010, b3);
+  const T R1_120 = x * R2_020;
+  const T R0_220 = fma(x, R1_120, R1_020);
+  const T R1_201 = z * R2_200;
+  const T R0_211 = y * R1_201;
+  const T R1_030 = fma(y, R2_020, T(2.0) * R2_010);
+  const T R0_130 = x * R1_030;
+  const T R1_021 = z * R2_020;
+  const T R0_121 = x * R1_021;
+  const T R0_040 = fma(y, R1_030, T(3.0) * R1_020);
+  const T R0_031 = z * R1_030;
+  const T R4_100 = x * b5;
+  const T R3_200 = fma(x, R4_100, b4);
+  const T R2_300 = fma(x, R3_200, T(2.0) * R3_100);
+  const T R1_400 = fma(x, R2_300, T(3.0) * R2_200);
+  const T R0_500 = fma(x, R1_400, T(4.0) * R1_300);
+  const T R0_410 = y * R1_400;
+  const T R0_401 = z * R1_400;
+  const T R4_010 = y * b5;
+  const T R3_020 = fma(y, R4_010, b4);
+  const T R2_120 = x * R3_020;
+  const T R1_220 = fma(x, R2_120, R2_020);
+  const T R0_320 = fma(x, R1_220, T(2.0) * R1_120);
+  const T R1_301 = z * R2_300;
+  const T R0_311 = y * R1_301;
+  const T R2_030 = fma(y, R3_020, T(2.0) * R3_010);
+  const T R1_130 = x * R2_030;
+  const T R0_230 = fma(x, R1_130, R1_030);
+  const T R0_221 = z * R1_220;
+  const T R1_040 = fma(y, R2_030, T(3.0) * R2_020);
+  const T R0_140 = x * R1_040;
+  const T R1_031 = z * R2_030;
+  const T R0_131 = x * R1_031;
+  const T R0_050 = fma(y, R1_040, T(4.0) * R1_030);
+  const T R0_041 = z * R1_040;
+  D[0] = b0;
+  D[1] = R0_100;
+  D[2] = R0_010;
+  D[3] = R0_001;
+  D[4] = R0_200;
+  D[5] = R0_110;
+  D[6] = R0_101;
+  D[7] = R0_020;
+  D[8] = R0_011;
+  D[10] = R0_300;
+  D[11] = R0_210;
+  D[12] = R0_201;
+  D[13] = R0_120;
+  D[14] = R0_111;
+  D[16] = R0_030;
+  D[17] = R0_021;
+  D[15] = -D[10] - D[13];
+  D[18] = -D[11] - D[16];
+  D[20] = R0_400;
+  D[21] = R0_310;
+  D[22] = R0_301;
+  D[23] = R0_220;
+  D[24] = R0_211;
+  D[26] = R0_130;
+  D[27] = R0_121;
+  D[30] = R0_040;
+  D[31] = R0_031;
+  D[25] = -D[20] - D[23];
+  D[28] = -D[21] - D[26];
+  D[32] = -D[23] - D[30];
+  D[35] = R0_500;
+  D[36] = R0_410;
+  D[37] = R0_401;
+  D[38] = R0_320;
+  D[39] = R0_311;
+  D[41] = R0_230;
+  D[42] = R0_221;
+  D[45] = R0_140;
+  D[46] = R0_131;
+  D[50] = R0_050;
+  D[51] = R0_041;
+  D[40] = -D[35] - D[38];
+  D[43] = -D[36] - D[41];
+  D[47] = -D[38] - D[45];
+  D[52] = -D[41] - D[50];
+}
+
+template <typename T> __device__ __forceinline__ void sfmm_uderivs_fold_5(T x, T y, T z, T rinv, T* D) {
+  const T R0_100 = x * T(-1.0);
+  const T R0_010 = y * T(-1.0);
+  const T R0_001 = z * T(-1.0);
+  const T R1_100 = x * T(3.0);
+  const T R0_200 = fma(x, R1_100, T(-1.0));
+  const T R1_010 = y * T(3.0);
+  const T R0_110 = x * R1_010;
+  const T R1_001 = z * T(3.0);
+  const T R0_101 = x * R1_001;
+  const T R0_020 = fma(y, R1_010, T(-1.0));
+  const T R0_011 = y * R1_001;
+  const T R2_100 = x * T(-15.0);
+  const T R1_200 = fma(x, R2_100, T(3.0));
+  const T R0_300 = fma(x, R1_200, T(2.0) * R1_100);
+  const T R0_210 = y * R1_200;
+  const T R0_201 = z * R1_200;
+  const T R2_010 = y * T(-15.0);
+  const T R1_020 = fma(y, R2_010, T(3.0));
+  const T R0_120 = x * R1_020;
+  const T R2_001 = z * T(-15.0);
+  const T R1_011 = y * R2_001;
+  const T R0_111 = x * R1_011;
+  const T R0_030 = fma(y, R1_020, T(2.0) * R1_010);
+  const T R0_021 = z * R1_020;
+  const T R3_100 = x * T(105.0);
+  const T R2_200 = fma(x, R3_100, T(-15.0));
+  const T R1_300 = fma(x, R2_200, T(2.0) * R2_100);
+  const T R0_400 = fma(x, R1_300, T(3.0) * R1_200);
+  const T R0_310 = y * R1_300;
+  const T R0_301 = z * R1_300;
+  const T R3_010 = y * T(105.0);
+  const T R2_020 = fma(y, R3_010, T(-15.0));
+  const T R1_120 = x * R2_020;
+  const T R0_220 = fma(x, R1_120, R1_020);
+  const T R1_201 = z * R2_200;
+  const T R0_211 = y * R1_201;
+  const T R1_030 = fma(y, R2_020, T(2.0) * R2_010);
+  const T R0_130 = x * R1_030;
+  const T R1_021 = z * R2_020;
+  const T R0_121 = x * R1_021;
+  const T R0_040 = fma(y, R1_030, T(3.0) * R1_020);
+  const T R0_031 = z * R1_030;
+  const T R4_100 = x * T(-945.0);
+  const T R3_200 = fma(x, R4_100, T(105.0));
+  const T R2_300 = fma(x, R3_200, T(2.0) * R3_100);
+  const T R1_400 = fma(x, R2_300, T(3.0) * R2_200);
+  const T R0_500 = fma(x, R1_400, T(4.0) * R1_300);
+  const T R0_410 = y * R1_400;
+  const T R0_401 = z * R1_400;
+  const T R4_010 = y * T(-945.0);
+  const T R3_020 = fma(y, R4_010, T(105.0));
+  const T R2_120 = x * R3_020;
+  const T R1_220 = fma(x, R2_120, R2_020);
+  const T R0_320 = fma(x, R1_220, T(2.0) * R1_120);
+  const T R1_301 = z * R2_300;
+  const T R0_311 = y * R1_301;
+  const T R2_030 = fma(y, R3_020, T(2.0) * R3_010);
+  const T R1_130 = x * R2_030;
+  const T R0_230 = fma(x, R1_130, R1_030);
+  const T R0_221 = z * R1_220;
+  const T R1_040 = fma(y, R2_030, T(3.0) * R2_020);
+  const T R0_140 = x * R1_040;
+  const T R1_031 = z * R2_030;
+  const T R0_131 = x * R1_031;
+  const T R0_050 = fma(y, R1_040, T(4.0) * R1_030);
+  const T R0_041 = z * R1_040;
+  T s = rinv;
+  D[0] = T(1.0) * s;
+  s = s * rinv;
+  D[1] = R0_100 * s;
+  D[2] = R0_010 * s;
+  D[3] = R0_001 * s;
+  s = s * rinv;
+  D[4] = R0_200 * s;
+  D[5] = R0_110 * s;
+  D[6] = R0_101 * s;
+  D[7] = R0_020 * s;
+  D[8] = R0_011 * s;
+  s = s * rinv;
+  D[10] = R0_300 * s;
+  D[11] = R0_210 * s;
+  D[12] = R0_201 * s;
+  D[13] = R0_120 * s;
+  D[14] = R0_111 * s;
+  D[16] = R0_030 * s;
+  D[17] = R0_021 * s;
+  D[15] = -D[10] - D[13];
+  D[18] = -D[11] - D[16];
+  s = s * rinv;
+  D[20] = R0_400 * s;
+  D[21] = R0_310 * s;
+  D[22] = R0_301 * s;
+  D[23] = R0_220 * s;
+  D[24] = R0_211 * s;
+  D[26] = R0_130 * s;
+  D[27] = R0_121 * s;
+  D[30] = R0_040 * s;
+  D[31] = R0_031 * s;
+  D[25] = -D[20] - D[23];
+  D[28] = -D[21] - D[26];
+  D[32] = -D[23] - D[30];
+  s = s * rinv;
+  D[35] = R0_500 * s;
+  D[36] = R0_410 * s;
+  D[37] = R0_401 * s;
+  D[38] = R0_320 * s;
+  D[39] = R0_311 * s;
+  D[41] = R0_230 * s;
+  D[42] = R0_221 * s;
+  D[45] = R0_140 * s;
+  D[46] = R0_131 * s;
+  D[50] = R0_050 * s;
+  D[51] = R0_041 * s;
+  D[40] = -D[35] - D[38];
+  D[43] = -D[36] - D[41];
+  D[47] = -D[38] - D[45];
+  D[52] = -D[41] - D[50];
+}
 

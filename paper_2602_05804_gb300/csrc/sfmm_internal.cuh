@@ -113,6 +113,7 @@ struct sfmm_ctx {
   DevBuf cf_arena, cf_off, cf_cnt, Tnode;  // shared walk: child frontiers, node coefficients
   DevBuf sym_own, sym_recv;               // walk mode 2: own and received sums per node (FP64)
   DevBuf wqueue;                          // walk mode 3: nodes in order of readiness
+  DevBuf src_rows;                        // shared walk: folded moments of every node (k_walk_prepare)
   // near field: chunks of long neighbour lists (extra work items, per-leaf
   // slot base, split leaves, partial sums) and the list entries in use
   DevBuf p2p_extra, p2p_split, p2p_slist, p2p_part;

@@ -33,6 +33,8 @@ struct WalkArgs {
   const float* Qf;
   const double* Qd;
   int nqs;  // row stride of Qf
+  const float* row32;   // source rows of the shared walk, by form (row_len)
+  const double* row64;
   const float4* prel;
   const double* px;
   const double* py;
@@ -74,6 +76,13 @@ template <int P> struct Exp;
     template <typename T> __device__ static void mono(T x, T y, T z, T* o) { sfmm_mono_##PP(x, y, z, o); }     \
     template <typename T> __device__ static void mono1(T x, T y, T z, T* o) { sfmm_mono_##PP1(x, y, z, o); }   \
     __device__ static const signed char* table() { return &sfmm_l2l_table_##PP[0][0]; }                       \
+    /* independent components (at most one z): source rows, sums, their unfolding */                           \
+    static constexpr int NR = SFMM_NR_##PP, NS = SFMM_NS_##PP, NX = SFMM_NX_##PP;                              \
+    template <typename T> __device__ static void fold(const T* Q, T* q) { sfmm_fold_##PP(Q, q); }              \
+    template <typename T> __device__ static void derivs_fold(T x, T y, T z, T ri, T* D) { sfmm_derivs_fold_##PP1(x, y, z, ri, D); } \
+    template <typename T> __device__ static void uderivs_fold(T x, T y, T z, T ri, T* D) { sfmm_uderivs_fold_##PP1(x, y, z, ri, D); } \
+    template <typename T> __device__ static void m2l_fold(const T* D, const T* q, T* C) { sfmm_m2l_fold_##PP(D, q, C); } \
+    __device__ static const signed char* unfold() { return &sfmm_unfold_##PP[0][0][0]; }                      \
   };
 SFMM_EXP(0, 1)
 SFMM_EXP(1, 2)
@@ -81,6 +90,25 @@ SFMM_EXP(2, 3)
 SFMM_EXP(3, 4)
 SFMM_EXP(4, 5)
 #undef SFMM_EXP
+
+// Source rows of the shared walk (k_walk_prepare), one per node.  FP32 form:
+// the folded moments about the node's centre, padded to float4.  FP64 form:
+// {centre (3), offset d to the centre of mass (3), folded moments about centre
+// + d}: the stored centre is the centre of mass to rounding, the rest of it is
+// the dipole.  With d = Q_1 / Q_0 carried beside the centre, and centre + d the
+// expansion centre of targets as well as sources (r, and with it every pair
+// force, antisymmetric), the dipole's 27 terms (p = 2) become six additions.
+template <int P, bool F32> __host__ __device__ constexpr int row_len() {
+  return F32 ? (Exp<P>::NR + 3) & ~3 : (6 + Exp<P>::NR + 1) & ~1;
+}
+
+// A node's expansion centre as centre + d: FP64 form of the shared walk (d = 0
+// where there are no rows).
+template <int P>
+__device__ __forceinline__ void node_offset(const WalkArgs& a, int v, double (&d)[3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) d[c] = a.row64 ? a.row64[(size_t)v * row_len<P, false>() + 3 + c] : 0.0;
+}
 
 // Reduce-scatter over the warp: on entry every lane holds v[0..32); on exit
 // v[0] on lane l is the warp sum of entry l.
@@ -98,6 +126,38 @@ __device__ __forceinline__ T reduce_scatter32(T (&v)[32], int lane) {
     }
   }
   return v[0];
+}
+
+// The same for N sums, 32 to a block: s[b] on lane l is the warp sum of entry
+// 32 b + l (a last block of fewer entries: entry 32 b + l mod the power of two
+// that holds them).
+template <int N, typename T>
+__device__ __forceinline__ void reduce_sums(const T (&C)[N], T* s, int lane) {
+#pragma unroll
+  for (int b = 0; b < (N + 31) / 32; ++b) {
+    const int left = N - 32 * b;
+    const int w = left >= 32 ? 32 : left > 16 ? 32 : left > 8 ? 16 : left > 4 ? 8 : left > 2 ? 4 : left;
+    T v[32];
+#pragma unroll
+    for (int t = 0; t < 32; ++t) v[t] = t < left ? C[32 * b + t < N ? 32 * b + t : 0] : T(0);
+#pragma unroll
+    for (int step = 0; step < 5; ++step) {
+      const int o = 16 >> step;
+      if (o < w) {
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int c = 0; c < o; ++c) {
+          const T send = upper ? v[c] : v[c + o];
+          const T keep = upper ? v[c + o] : v[c];
+          v[c] = keep + __shfl_xor_sync(SFMM_FULL, send, o);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      if (o >= w) v[0] += __shfl_xor_sync(SFMM_FULL, v[0], o);
+    s[b] = v[0];
+  }
 }
 
 // Acceptance test of Sect. 3: accept iff (l_t + l_s) < theta d and not
@@ -172,6 +232,95 @@ __device__ __forceinline__ void m2l_eval(int s, const float4& hiA, const float4&
     for (int t = 0; t < E::NQ; ++t) Q[t] = __ldg(q + t);
     E::m2l(D, Q, C);
   }
+}
+
+// One interaction on the independent components (see gen_expansion.py) added
+// to the lane's sums: 41 FP64 instructions against 121 at p = 2 for the
+// contraction, 35 against 52 for the derivatives.  FP32 form: r = s_B - s_A
+// from the acceptance test.  FP64 form: from the rows; the derivatives take
+// powers of 1/r itself while they stay in range, else r scaled by a power of
+// two.
+template <int P, bool F32>
+__device__ __forceinline__ void m2l_fold(int s, double cAx, double cAy, double cAz, const double (&dA)[3],
+                                         const WalkArgs& a, typename std::conditional<F32, float, double>::type* C,
+                                         const float4& r) {
+  using E = Exp<P>;
+  if (s < 0) return;
+  constexpr int RL = row_len<P, F32>();
+  if constexpr (F32) {
+    float q[RL];
+    const float4* q4 = reinterpret_cast<const float4*>(a.row32) + (size_t)s * (RL / 4);
+#pragma unroll
+    for (int t = 0; t < RL / 4; ++t) {
+      const float4 v = __ldg(q4 + t);
+      q[4 * t] = v.x;
+      q[4 * t + 1] = v.y;
+      q[4 * t + 2] = v.z;
+      q[4 * t + 3] = v.w;
+    }
+    const float ri = rsqrtf(fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z)));
+    float D[E::NMONO1];
+    E::uderivs_fold(r.x * ri, r.y * ri, r.z * ri, ri, D);
+    E::m2l_fold(D, q, C);
+  } else {
+    double q[RL];
+    const double2* q2 = reinterpret_cast<const double2*>(a.row64) + (size_t)s * (RL / 2);
+#pragma unroll
+    for (int t = 0; t < RL / 2; ++t) {
+      const double2 v = __ldg(q2 + t);
+      q[2 * t] = v.x;
+      q[2 * t + 1] = v.y;
+    }
+    double rx = (q[0] - cAx) + (q[3] - dA[0]), ry = (q[1] - cAy) + (q[4] - dA[1]), rz = (q[2] - cAz) + (q[5] - dA[2]);
+    double r2 = fma(rx, rx, fma(ry, ry, rz * rz));
+    double D[E::NMONO1];
+    if (r2 >= 0x1p-110 && r2 <= 0x1p110) {
+      E::derivs_fold(rx, ry, rz, rsqrt_refined(r2), D);
+    } else {
+      // D(r) = k^(|gamma|+1) D(k r), k a power of two that brings r near 1
+      const int e = ilogb(fmax(fmax(fabs(rx), fabs(ry)), fabs(rz)));
+      const double k = ldexp(1.0, -e);
+      rx *= k;
+      ry *= k;
+      rz *= k;
+      r2 = fma(rx, rx, fma(ry, ry, rz * rz));
+      E::derivs_fold(rx, ry, rz, rsqrt(r2), D);
+      double w = k;
+#pragma unroll
+      for (int n = 0, t = 0; n <= P + 1; ++n) {
+#pragma unroll
+        for (; t < ncoef(n); ++t) D[t] *= w;
+        w *= k;
+      }
+    }
+    E::m2l_fold(D, q + 6, C);
+  }
+}
+
+// Sums of one node (reduce_sums) to its coefficient vector, entry lane + 32 b
+// in lev[b]: each is a sum of a few of them.  sx: scratch of 32 (NS blocks).
+template <int P, typename R>
+__device__ __forceinline__ void unfold_sums(const R* sums, R* lev, R* sx, const signed char* s_unf, int lane) {
+  using E = Exp<P>;
+  constexpr int NB = (E::NS + 31) / 32, NCS = (E::NC + 31) / 32;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) sx[32 * b + lane] = sums[b];
+  __syncwarp();
+#pragma unroll
+  for (int b = 0; b < NCS; ++b) {
+    const int j = lane + 32 * b;
+    R v = R(0);
+    if (j < E::NC) {
+      const signed char* u = s_unf + j * 2 * E::NX;
+#pragma unroll
+      for (int t = 0; t < E::NX; ++t) {
+        const int f = u[2 * t + 1];
+        if (f != 0) v = fma(R(f), sx[u[2 * t]], v);
+      }
+    }
+    lev[b] = v;
+  }
+  __syncwarp();
 }
 
 // Sign (-1)^|gamma| of entry t of a derivative vector (entries are ordered by

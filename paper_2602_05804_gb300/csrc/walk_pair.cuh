@@ -108,9 +108,11 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? 4 : 1) k_walk_pair(
   __shared__ R s_T[WALK_WARPS][NCS * 32];
   __shared__ R s_h[WALK_WARPS][E::NMONO1];
   __shared__ signed char s_tab[NC * NC];
+  __shared__ signed char s_unf[NC * 2 * E::NX];
   {
-    const signed char* tab = E::table();
+    const signed char *tab = E::table(), *unf = E::unfold();
     for (int t = threadIdx.x; t < NC * NC; t += WALK_NT) s_tab[t] = tab[t];
+    for (int t = threadIdx.x; t < NC * 2 * E::NX; t += WALK_NT) s_unf[t] = unf[t];
   }
   __syncthreads();
 
@@ -317,22 +319,29 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? 4 : 1) k_walk_pair(
         st_m2l += (unsigned long long)k.nacc * la.nlu[k.A];
       }
       // its batches, in the order they filled
-      R C[NCS * 32];
+      R C[E::NS];
 #pragma unroll
-      for (int t = 0; t < NCS * 32; ++t) C[t] = R(0);
+      for (int t = 0; t < E::NS; ++t) C[t] = R(0);
       const int* const bat = bat_of(q);
-      for (int b = 0; b < k.nb; b += 32) m2l_eval<P, F32>(bat[b + lane], k.hi, k.lo, k.cx, k.cy, k.cz, a, C);
+      double dA[3] = {0.0, 0.0, 0.0};
+      if constexpr (!F32) node_offset<P>(a, k.A, dA);
+      for (int b = 0; b < k.nb; b += 32) {
+        const int s = bat[b + lane];
+        float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (F32 && s >= 0) {
+          const float4 hB = a.geo_hi[s], lB = a.geo_lo[s];
+          r.x = df_diff(hB.x, lB.x, k.hi.x, k.lo.x);
+          r.y = df_diff(hB.y, lB.y, k.hi.y, k.lo.y);
+          r.z = df_diff(hB.z, lB.z, k.hi.z, k.lo.z);
+        }
+        m2l_fold<P, F32>(s, k.cx, k.cy, k.cz, dA, a, C, r);
+      }
       // coefficients: own sums plus the parent's, translated; an internal
       // child stores them and hands its children on, a leaf evaluates them
       // (L2P) and writes its neighbour list
-      R lev[NCS];
-#pragma unroll
-      for (int b = 0; b < NCS; ++b) {
-        R v[32];
-#pragma unroll
-        for (int t = 0; t < 32; ++t) v[t] = C[32 * b + t];
-        lev[b] = reduce_scatter32(v, lane);
-      }
+      R sums[(E::NS + 31) / 32], lev[NCS];
+      reduce_sums(C, sums, lane);
+      unfold_sums<P>(sums, lev, s_T[warp], s_unf, lane);
       R Tn[NCS];
       float Tl[NCS];
       const bool leafA = k.r < 0;
@@ -382,11 +391,4 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? 4 : 1) k_walk_pair(
     atomicAdd(&a.stat[2], st_pl);
     atomicAdd(&a.stat[4], (unsigned long long)st_fb);
   }
-}
-
-// Queue of the pair walk: the system roots fill the first slots.
-__global__ void k_queue_seed_pairs(int nsys, const int* __restrict__ sys_root, int* __restrict__ queue,
-                                   int* __restrict__ tail) {
-  for (int i = threadIdx.x; i < nsys; i += blockDim.x) queue[i] = 2 * sys_root[i] + 1;
-  if (threadIdx.x == 0) *tail = nsys;
 }

@@ -12,6 +12,9 @@
 // (T(A) = shift(T(parent)) + C(A), Eq. gravmtranslat) and evaluated at the
 // leaves (L2P).  Leaves run the lowering of Algorithm 2 and emit their
 // neighbour lists exactly as in the per-leaf replay.
+#include <algorithm>
+
+#include "mom_ops.cuh"
 #include "walk_common.cuh"
 
 namespace sfmm {
@@ -110,9 +113,12 @@ __device__ __forceinline__ void node_coefficients(const LevelArgs& la, int A, in
         hy = df_diff(hiA.y, loA.y, hiP.y, loP.y);
         hz = df_diff(hiA.z, loA.z, hiP.z, loP.z);
       } else {
-        hx = cAx - a.ncx[par];
-        hy = cAy - a.ncy[par];
-        hz = cAz - a.ncz[par];
+        double dA[3], dP[3];
+        node_offset<P>(a, A, dA);
+        node_offset<P>(a, par, dP);
+        hx = (cAx - a.ncx[par]) + (dA[0] - dP[0]);
+        hy = (cAy - a.ncy[par]) + (dA[1] - dP[1]);
+        hz = (cAz - a.ncz[par]) + (dA[2] - dP[2]);
       }
       R hm[E::NMONO1];
       E::mono1(hx, hy, hz, hm);
@@ -177,6 +183,8 @@ __device__ __forceinline__ void leaf_l2p(const LevelArgs& la, int A, double cAx,
     else sT[lane + 32 * b] = Tn[b];
   }
   __syncwarp();
+  double dA[3] = {0.0, 0.0, 0.0};
+  if constexpr (!F32) node_offset<P>(a, A, dA);
   for (int t = lane; t < nL; t += 32) {
     const int i = fL + t;
     R ax, ay, az;
@@ -186,9 +194,9 @@ __device__ __forceinline__ void leaf_l2p(const LevelArgs& la, int A, double cAx,
       ay = p.y;
       az = p.z;
     } else {
-      ax = a.px[i] - cAx;
-      ay = a.py[i] - cAy;
-      az = a.pz[i] - cAz;
+      ax = (a.px[i] - cAx) - dA[0];
+      ay = (a.py[i] - cAy) - dA[1];
+      az = (a.pz[i] - cAz) - dA[2];
     }
     R am[E::NQ], o4[4];
     E::mono(ax, ay, az, am);
@@ -222,9 +230,14 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
   __shared__ R s_T[WALK_WARPS][NCS * 32];
   __shared__ R s_h[WALK_WARPS][E::NMONO1];
   __shared__ signed char s_tab[NC * NC];
+  __shared__ signed char s_unf[SYM ? 1 : NC * 2 * E::NX];
   {
     const signed char* tab = E::table();
     for (int t = threadIdx.x; t < NC * NC; t += WALK_NT) s_tab[t] = tab[t];
+    if constexpr (!SYM) {
+      const signed char* unf = E::unfold();
+      for (int t = threadIdx.x; t < NC * 2 * E::NX; t += WALK_NT) s_unf[t] = unf[t];
+    }
   }
   __syncthreads();
 
@@ -310,11 +323,12 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
     bool two_leaves = false;
     if (queue && !leafA) two_leaves = a.nright[A + 1] < 0 && a.nright[rA] < 0;
     const float4 hiA = a.geo_hi[A], loA = a.geo_lo[A];
-    double cAx = 0.0, cAy = 0.0, cAz = 0.0;
-    if (!F32) {
+    double cAx = 0.0, cAy = 0.0, cAz = 0.0, dA[3] = {0.0, 0.0, 0.0};
+    if constexpr (!F32) {
       cAx = a.ncx[A];
       cAy = a.ncy[A];
       cAz = a.ncz[A];
+      if constexpr (!SYM) node_offset<P>(a, A, dA);
     }
     // the opened list inherited from the parent (a system's root starts from
     // itself), read in order; a leaf's lowering pushes the pairs it opens on
@@ -346,9 +360,10 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
       }
       cfw = la.cf_out + cfbase;
     }
-    R C[NCS * 32];
+    constexpr int NSUM = SYM ? NCS * 32 : E::NS;
+    R C[NSUM];
 #pragma unroll
-    for (int t = 0; t < NCS * 32; ++t) C[t] = R(0);
+    for (int t = 0; t < NSUM; ++t) C[t] = R(0);
     int nq = 0, nacc_tot = 0;
     int rankA = 0;
     R QA[SYM ? (F32 ? ((E::NQ + 3) / 4) * 4 : E::NQ) : 1];
@@ -482,7 +497,7 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
             st_m2l_p += (unsigned long long)la.nlu[src];
           }
         } else {
-          m2l_eval<P, F32>(src, hiA, loA, cAx, cAy, cAz, a, C, rq);
+          m2l_fold<P, F32>(src, cAx, cAy, cAz, dA, a, C, rq);
         }
         nq -= take;
       }
@@ -505,12 +520,18 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
 
     // coefficients of A: own level sum plus the parent's, translated
     R lev[NCS];
+    if constexpr (SYM) {
 #pragma unroll
-    for (int b = 0; b < NCS; ++b) {
-      R v[32];
+      for (int b = 0; b < NCS; ++b) {
+        R v[32];
 #pragma unroll
-      for (int t = 0; t < 32; ++t) v[t] = C[32 * b + t];
-      lev[b] = reduce_scatter32(v, lane);
+        for (int t = 0; t < 32; ++t) v[t] = C[32 * b + t];
+        lev[b] = reduce_scatter32(v, lane);
+      }
+    } else {
+      R sums[(E::NS + 31) / 32];
+      reduce_sums(C, sums, lane);
+      unfold_sums<P>(sums, lev, s_T[warp], s_unf, lane);
     }
     R Tn[NCS];
     float Tl[NCS];
@@ -637,11 +658,67 @@ __global__ void __launch_bounds__(WALK_NT) k_walk_finalize(const LevelArgs la, i
   }
 }
 
-// Queue walk: the system roots (no walk parent) fill the first slots.
-__global__ void k_queue_seed(int nsys, const int* __restrict__ sys_root, long long* __restrict__ queue,
-                             int* __restrict__ tail) {
-  for (int i = threadIdx.x; i < nsys; i += blockDim.x) queue[i] = (long long)(unsigned)sys_root[i];
-  if (threadIdx.x == 0) *tail = nsys;
+// Before the shared walk: every node's source row, and (queue walks) the empty
+// queue with the system roots in its first slots.  pairs: a root's item is
+// 2 root + 1 in the pair queue.
+template <int P, bool F32>
+__global__ void __launch_bounds__(128) k_walk_prepare(const LevelArgs la, const float* __restrict__ Qf,
+                                                      const double* __restrict__ Qd, float* __restrict__ row32,
+                                                      double* __restrict__ row64, bool pairs,
+                                                      const int* __restrict__ sys_root) {
+  using E = Exp<P>;
+  constexpr int RL = row_len<P, F32>();
+  const WalkArgs& a = la.w;
+  const int nn = (int)la.counts[0];
+  const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  for (int v = t0; v < nn; v += nt) {
+    if constexpr (F32) {
+      float Q[E::NQ], q[RL];
+#pragma unroll
+      for (int t = 0; t < E::NQ; ++t) Q[t] = Qf[(size_t)v * a.nqs + t];
+#pragma unroll
+      for (int t = E::NR; t < RL; ++t) q[t] = 0.0f;
+      E::fold(Q, q);
+      float4* out = reinterpret_cast<float4*>(row32) + (size_t)v * (RL / 4);
+#pragma unroll
+      for (int t = 0; t < RL / 4; ++t) out[t] = make_float4(q[4 * t], q[4 * t + 1], q[4 * t + 2], q[4 * t + 3]);
+    } else {
+      double Q[E::NQ], S[E::NQ], q[RL];
+#pragma unroll
+      for (int t = 0; t < E::NQ; ++t) {
+        Q[t] = Qd[(size_t)v * E::NQ + t];
+        S[t] = 0.0;
+      }
+      double d[3] = {0.0, 0.0, 0.0};
+      if constexpr (P >= 1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = Q[1 + c] / Q[0];
+        double g[E::NQ];
+        E::mono(-d[0], -d[1], -d[2], g);
+        MomOps<P>::m2m(g, Q, S);  // moments about centre + d (Eq. massmomtrans)
+      } else {
+        S[0] = Q[0];
+      }
+      q[RL - 1] = 0.0;
+      q[0] = a.ncx[v];
+      q[1] = a.ncy[v];
+      q[2] = a.ncz[v];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) q[3 + c] = d[c];
+      E::fold(S, q + 6);
+      double2* out = reinterpret_cast<double2*>(row64) + (size_t)v * (RL / 2);
+#pragma unroll
+      for (int t = 0; t < RL / 2; ++t) out[t] = make_double2(q[2 * t], q[2 * t + 1]);
+    }
+  }
+  if (la.queue) {
+    const int bound = nn + 1 - (int)la.counts[1];
+    for (int i = t0; i < bound; i += nt) {
+      if (pairs) la.queue[i] = i < la.nsys ? 2 * sys_root[i] + 1 : -1;
+      else la.queue64[i] = i < la.nsys ? (long long)(unsigned)sys_root[i] : -1LL;
+    }
+    if (t0 == 0) *la.q_tail = la.nsys;
+  }
 }
 
 template <int P, bool F32, bool SYM>
@@ -674,8 +751,8 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
     int l2 = 0;
     if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device) != cudaSuccess) l2 = 0;
     // geometry and right child (36 B), list offset and count (12 B),
-    // moments, coefficients
-    const size_t mom = F32 ? 4 * (size_t)((ncoef(order) + 3) & ~3) : 24 + 8 * (size_t)E::NQ;
+    // source row, coefficients
+    const size_t mom = (F32 ? 4 : 8) * (size_t)row_len<P, F32>();
     const size_t per_node = 48 + mom + 8 * (size_t)tstride;
     sched = ((double)per_node * nn <= 2.0 * (double)l2) ? 2 : 3;
   }
@@ -779,6 +856,8 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
     la.Cown = SYM ? c->sym_own.as<double>() : nullptr;
     la.Erecv = SYM ? c->sym_recv.as<double>() : nullptr;
     la.queue = nullptr;
+    la.counts = c->d_counts;
+    la.nsys = c->nsys;
     if (queue) {
       // one launch: a warp takes the next slot of the queue and waits until
       // the item there has been pushed.  Node queue: the system roots first,
@@ -793,16 +872,22 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
       la.queue64 = c->wqueue.as<long long>();
       la.q_head = reinterpret_cast<int*>(ctr + 14);
       la.q_tail = reinterpret_cast<int*>(ctr + 15);
-      la.counts = c->d_counts;
-      la.nsys = c->nsys;
-      SFMM_CUDA_TRY(cudaMemsetAsync(la.queue, 0xff, (pairs ? sizeof(int) : sizeof(long long)) * (size_t)q_bound,
-                                    c->stream));
-      if (pairs) k_queue_seed_pairs<<<1, 32, 0, c->stream>>>(c->nsys, c->sys_root.as<int>(), la.queue, la.q_tail);
-      else k_queue_seed<<<1, 32, 0, c->stream>>>(c->nsys, c->sys_root.as<int>(), la.queue64, la.q_tail);
       la.level = 0;
       la.level_nodes = nullptr;
       la.level_begin = 0;
       la.level_count = la.q_total;
+    }
+    if constexpr (!SYM) {
+      if ((rc = c->src_rows.ensure((F32 ? sizeof(float) : sizeof(double)) * row_len<P, F32>() * (size_t)nn_b))) return rc;
+      la.w.row32 = c->src_rows.as<float>();
+      la.w.row64 = c->src_rows.as<double>();
+      const int blocks = std::max(1, std::min((nn_b + 127) / 128, 16 * num_sms(c->device)));
+      k_walk_prepare<P, F32><<<blocks, 128, 0, c->stream>>>(la, a.Qf, a.Qd, c->src_rows.as<float>(),
+                                                            c->src_rows.as<double>(), pairs, c->sys_root.as<int>());
+      ++c->nlaunch;
+      SFMM_CUDA_TRY(cudaGetLastError());
+    }
+    if (queue) {
       if (la.q_total > 0 || c->graph_mode) {
         // one block per resident slot (the queue needs none resident: a warp
         // only takes a slot while it runs, and a node's parent always holds
@@ -811,7 +896,6 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
         else k_walk_level<P, F32, false, true><<<q_blocks, WALK_NT, 0, c->stream>>>(la);
         ++c->nlaunch;
       }
-      ++c->nlaunch;
       SFMM_CUDA_TRY(cudaGetLastError());
     }
     // internal nodes level by level (each needs its parent's opened list and
