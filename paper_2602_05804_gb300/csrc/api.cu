@@ -445,7 +445,6 @@ int sfmm_gravity(sfmm_ctx* c, double theta, int order, double* acc, double* pot)
     if (c->profile) cudaEventRecord(c->ev[5], st);
     double* red = nullptr;
     if ((rc = run_reduce(c, &red))) return set_error(c, rc, "reduction failed");
-    if (c->nsys > 1 && (rc = run_reduce_systems(c))) return set_error(c, rc, "reduction failed");
     if (c->profile) cudaEventRecord(c->ev[6], st);
     cudaError_t e = cudaMemcpyAsync(c->h_scalars + 16, red, 5 * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess)  // walk counters (statistics, buffer needs) and pair evaluations
@@ -532,7 +531,6 @@ int issue_step(sfmm_ctx* c, const double* pos, const double* mass, const double*
   if ((rc = run_p2p(c, acc, pot))) return rc;
   double* red = nullptr;
   if ((rc = run_reduce(c, &red))) return rc;
-  if (c->nsys > 1 && (rc = run_reduce_systems(c))) return rc;
   SFMM_CUDA_TRY(cudaMemcpyAsync(c->h_scalars + 16, red, 5 * sizeof(double), cudaMemcpyDeviceToHost, st));
   SFMM_CUDA_TRY(cudaMemcpyAsync(c->h_scalars + 32, c->counters.p, 20 * sizeof(unsigned long long),
                                 cudaMemcpyDeviceToHost, st));

@@ -174,8 +174,7 @@ int run_walk(sfmm_ctx* c, double theta, int order, bool dump, int64_t cap_m2l, i
 
 // p2p.cu
 int run_p2p(sfmm_ctx* c, double* acc, double* pot);
-int run_reduce(sfmm_ctx* c, double** out_dev);  // device pointer of the 5 sums
-int run_reduce_systems(sfmm_ctx* c);             // per-system sums (batches)
+int run_reduce(sfmm_ctx* c, double** out_dev);  // device pointer of the 5 sums; batches: also per system
 
 // autotune.cu
 void tune_table_free(sfmm_ctx* c);
