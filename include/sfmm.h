@@ -126,7 +126,9 @@ int sfmm_set_stream(sfmm_ctx* ctx, void* stream);
  *                    systems only, sfmm_build_batch returns ENOTIMPL)
  *   "p2p_chunk"      neighbour-list entries per near-field work item: longer
  *                    lists are cut into chunks evaluated as separate items
- *                    and recombined in chunk order (default 256, 32..65536)
+ *                    and recombined in chunk order (default 256, 32..65536;
+ *                    fewer are taken, down to 8, when all lists together are
+ *                    too short to occupy the GPU)
  *   "p2p_blocks"     near-field blocks per SM (0, default: as many as fit)
  *   "autotune_theta", "autotune_order"  theta and order that autotuned leaf
  *                    sizes are chosen for (sfmm_build_batch with NULL sizes)

@@ -59,10 +59,20 @@ struct P2PArgs {
   const int* slist;   // the split leaves
   void* part;         // [slot][lmax][4] partial sums in the form's type
   int lmax;
-  int chunk;          // neighbour-list entries per work item of a split list
+  unsigned long long* chunk_now;  // the entries taken (p2p_chunk_of, written by the split pass)
   unsigned long long* pair_counter;  // pair evaluations (statistics)
   const int* items;   // FP64 form: the work items k_p2p_fexp left, items[-4] of them
 };
+
+// Neighbour-list entries per work item: the option's value, fewer when the
+// lists are too few for eight items per resident warp, down to 8 entries (an
+// item then stages about a warp's width of sources a few times).  With 256
+// entries throughout, the near field of 1000 particles took 54 us in 96 items
+// and that of 13,000 in the FP64 form 4.9 ms in 2500 items on 2432 warps.
+__host__ __device__ __forceinline__ int p2p_chunk_of(unsigned long long total, int most, int want) {
+  const unsigned long long c = total / (unsigned)want;
+  return c >= (unsigned long long)most ? most : (c < 8 ? 8 : (int)c);
+}
 
 // M4 softening kernel of one particle (compact support 2h): g = phi'(r)/r
 // and phi, -> 1/r^3 and -1/r outside 2h.  Both pieces' polynomials are
@@ -254,8 +264,13 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
     R ax0 = R(0), ay0 = R(0), az0 = R(0), pt0 = R(0);
     R ax1 = R(0), ay1 = R(0), az1 = R(0), pt1 = R(0);
 
-    const long long off = a.p2p_off[leaf] + (long long)chunk * a.chunk;
-    const int cnt = (pslot < 0) ? a.p2p_cnt[leaf] : min(a.chunk, a.p2p_cnt[leaf] - chunk * a.chunk);
+    long long off = a.p2p_off[leaf];
+    int cnt = a.p2p_cnt[leaf];
+    if (pslot >= 0) {
+      const int per = (int)*a.chunk_now;
+      off += (long long)chunk * per;
+      cnt = min(per, cnt - chunk * per);
+    }
     int nfar = 0, nnear = 0;
     int e = 0;                 // next list entry to load
     int tot = 0, pdone = 0;    // particles of the loaded entries / staged so far
@@ -644,7 +659,10 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
 __global__ void k_p2p_split(const uint32_t* __restrict__ counts, const int* __restrict__ p2p_cnt,
                             int* __restrict__ split, int2* __restrict__ extra, int* __restrict__ slist,
                             unsigned long long* __restrict__ ctr, int max_extra, int max_slots, int max_split,
-                            int chunk, int* __restrict__ status) {
+                            int most, int want, const unsigned long long* __restrict__ list_total,
+                            unsigned long long* __restrict__ chunk_now, int* __restrict__ status) {
+  const int chunk = p2p_chunk_of(*list_total, most, want);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *chunk_now = (unsigned long long)chunk;
   const int nleaves = (int)counts[1];
   for (int leaf = blockIdx.x * blockDim.x + threadIdx.x; leaf < nleaves; leaf += gridDim.x * blockDim.x) {
     const int cnt = p2p_cnt[leaf];
@@ -673,6 +691,7 @@ __global__ void k_p2p_split(const uint32_t* __restrict__ counts, const int* __re
 template <bool F32>
 __global__ void k_p2p_combine(const P2PArgs a) {
   const int nsplit = (int)a.d_split[2];
+  const int chunk = (int)*a.chunk_now;
   using R = typename std::conditional<F32, float, double>::type;
   const int lane = threadIdx.x & 31;
   const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -680,7 +699,7 @@ __global__ void k_p2p_combine(const P2PArgs a) {
     const int leaf = a.slist[q];
     const int L = a.leaf_node[leaf];
     const int fL = a.nfirst[L], nL = a.ncount[L];
-    const int nch = (a.p2p_cnt[leaf] + a.chunk - 1) / a.chunk;
+    const int nch = (a.p2p_cnt[leaf] + chunk - 1) / chunk;
     const int base = a.split[leaf];
     for (int t = lane; t < nL; t += 32) {
       R v[4] = {R(0), R(0), R(0), R(0)};
@@ -692,6 +711,15 @@ __global__ void k_p2p_combine(const P2PArgs a) {
       p2p_finish<F32>(a, fL + t, v);
     }
   }
+}
+
+int p2p_blocks_fit(sfmm_ctx* c) {
+  const bool f32 = (c->precision == SFMM_FP32);
+  const int nt = 32 * p2p_warps<true>();
+  int per_sm = 0;
+  if (f32) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<true>, nt, 0);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_fexp, FX_NT, 0);
+  return per_sm < 1 ? 1 : per_sm;
 }
 
 int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
@@ -707,14 +735,23 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   unsigned long long* ctr = c->counters.as<unsigned long long>();
   SFMM_CUDA_TRY(cudaMemsetAsync(ctr + 10, 0, 4 * sizeof(unsigned long long), c->stream));
   const bool f32 = (c->precision == SFMM_FP32);
+  // the grids: one block per resident slot
+  const int nt = 32 * (f32 ? p2p_warps<true>() : p2p_warps<false>());
+  const int fit = p2p_blocks_fit(c);
+  const int per_sm = (c->p2p_blocks > 0 && c->p2p_blocks < fit) ? c->p2p_blocks : fit;  // option: fewer
+  const int nblocks = per_sm * num_sms(c->device);
+  const int want = 8 * nblocks * (f32 ? p2p_warps<true>() : FX_WARPS);
   // long lists: slots, extra items and split leaves are counted by the split
   // pass on the device; the buffers are sized from bounds on the host (a list
-  // of cnt > chunk entries takes ceil(cnt / chunk) <= 2 cnt / chunk slots, so
-  // all of them fit 2 arena / chunk), with no wait for the walk
+  // of cnt > chunk entries takes ceil(cnt / chunk) <= 2 cnt / chunk slots, and
+  // entries / chunk is at most arena / option or 9/8 want), with no wait for
+  // the walk
   const int64_t arena_cap = (int64_t)(c->arena.bytes / sizeof(int));
-  const int nslots = (int)std::min<int64_t>(2 * arena_cap / c->p2p_chunk + 2, INT32_MAX / 2);
-  const int nsplit =
-      (int)std::min<int64_t>(std::min<int64_t>(c->graph_mode ? c->n : nl, arena_cap / (c->p2p_chunk + 1) + 1), nslots);
+  const int nslots =
+      (int)std::min<int64_t>(std::max<int64_t>(2 * arena_cap / c->p2p_chunk, 3 * (int64_t)want) + 2, INT32_MAX / 2);
+  const int nsplit = (int)std::min<int64_t>(
+      std::min<int64_t>(c->graph_mode ? c->n : nl, std::max<int64_t>(arena_cap / (c->p2p_chunk + 1), 2 * (int64_t)want) + 1),
+      nslots);
   const int nextra = nslots;
   int lmax = c->leaf_size;
   for (int v : c->h_sys_lsz) lmax = v > lmax ? v : lmax;
@@ -726,7 +763,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   const int sblocks = std::max(1, std::min((nl_b + 255) / 256, 8 * num_sms(c->device)));
   k_p2p_split<<<sblocks, 256, 0, c->stream>>>(c->d_counts, c->p2p_cnt.as<int>(), c->p2p_split.as<int>(),
                                                      c->p2p_extra.as<int2>(), c->p2p_slist.as<int>(), ctr + 11,
-                                                     nextra, nslots, nsplit, c->p2p_chunk, c->d_status);
+                                                     nextra, nslots, nsplit, c->p2p_chunk, want, ctr + 9, ctr + 7, c->d_status);
   ++c->nlaunch;
   SFMM_CUDA_TRY(cudaGetLastError());
   P2PArgs a{};
@@ -763,15 +800,8 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   a.slist = c->p2p_slist.as<int>();
   a.part = c->p2p_part.p;
   a.lmax = lmax;
-  a.chunk = c->p2p_chunk;
+  a.chunk_now = ctr + 7;
   a.pair_counter = ctr + 3;
-  const int nt = 32 * (f32 ? p2p_warps<true>() : p2p_warps<false>());
-  int per_sm = 0;
-  if (f32) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<true>, nt, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<false>, nt, 0);
-  if (per_sm < 1) per_sm = 1;
-  if (c->p2p_blocks > 0 && c->p2p_blocks < per_sm) per_sm = c->p2p_blocks;  // option: fewer blocks per SM
-  const int nblocks = per_sm * num_sms(c->device);
   if (f32) {
     k_p2p<true><<<nblocks, nt, 0, c->stream>>>(a);
   } else {
@@ -794,14 +824,10 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
     f.fb = c->fx_items.as<int>();
     k_fexp_records<<<(int)std::min<size_t>((n + 255) / 256, 8 * (size_t)num_sms(c->device)), 256, 0, c->stream>>>(
         a, f, (int)n);
-    int fx_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fx_sm, k_p2p_fexp, FX_NT, 0);
-    fx_sm = std::max(1, fx_sm);
-    if (c->p2p_blocks > 0 && c->p2p_blocks < fx_sm) fx_sm = c->p2p_blocks;
-    k_p2p_fexp<<<fx_sm * num_sms(c->device), FX_NT, 0, c->stream>>>(a, f);
+    k_p2p_fexp<<<nblocks, FX_NT, 0, c->stream>>>(a, f);
     a.leaf_counter = f.fb + 1;
     a.items = f.fb + 4;
-    k_p2p<false><<<nblocks, nt, 0, c->stream>>>(a);
+    k_p2p<false><<<num_sms(c->device), nt, 0, c->stream>>>(a);
     c->nlaunch += 2;
   }
   ++c->nlaunch;
@@ -815,15 +841,6 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
     SFMM_CUDA_TRY(cudaGetLastError());
   }
   return SFMM_OK;
-}
-
-int p2p_blocks_fit(sfmm_ctx* c) {
-  const bool f32 = (c->precision == SFMM_FP32);
-  const int nt = 32 * p2p_warps<true>();
-  int per_sm = 0;
-  if (f32) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<true>, nt, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_fexp, FX_NT, 0);
-  return per_sm < 1 ? 1 : per_sm;
 }
 
 }  // namespace sfmm

@@ -107,6 +107,8 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
   __shared__ __align__(16) float s_part[FX_WARPS][12][32];  // run sums; softened results (32 x 4 doubles)
   __shared__ int s_qj[FX_WARPS][FX_SQ];  // queued softened pairs: source particle, target in the leaf
   __shared__ unsigned char s_qt[FX_WARPS][FX_SQ];
+  __shared__ unsigned s_gm[FX_WARPS][32];  // a batch's targets: lanes holding their results, target in the leaf
+  __shared__ unsigned char s_gt[FX_WARPS][32];
   __shared__ float2 s_bias[FX_WARPS][32];  // per target of a group: level-0 bias of force and potential
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -155,8 +157,13 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
     for (int t = lane; t < nL * 4; t += 32) (&s_acc[warp][0][0])[t] = 0.0;
     __syncwarp();
 
-    const long long off = a.p2p_off[leaf] + (long long)chunk * a.chunk;
-    const int cnt = (pslot < 0) ? a.p2p_cnt[leaf] : min(a.chunk, a.p2p_cnt[leaf] - chunk * a.chunk);
+    long long off = a.p2p_off[leaf];
+    int cnt = a.p2p_cnt[leaf];
+    if (pslot >= 0) {
+      const int per = (int)*a.chunk_now;
+      off += (long long)chunk * per;
+      cnt = min(per, cnt - chunk * per);
+    }
     int ns = 0;                // staged sources
     int e = 0;                 // next list entry to load
     int tot = 0, pdone = 0;    // particles of the loaded entries / staged so far
@@ -168,8 +175,7 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
     // target: above, and below from the sources outside every kernel
     float bf = 0.0f, bp = 0.0f, low = 0.0f;
 
-    // queued softened pairs, the last cnt entries, one per lane; the lowest
-    // lane of each target adds the target's results in lane order
+    // queued softened pairs, the last cnt entries, one per lane
     auto soft_batch = [&](int base, int nb) {
       double4_16a* const res = reinterpret_cast<double4_16a*>(&s_part[warp][0][0]);
       const int t = lane < nb ? (int)s_qt[warp][base + lane] : 64 + lane;
@@ -188,24 +194,27 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
         const double mg = -mh * g;
         v = make_double4_16a(mg * dx, mg * dy, mg * dz, mh * phi);
       }
+      // each target's results in lane order, one (target, component) per lane:
+      // 8 targets at a time
       const unsigned same = __match_any_sync(SFMM_FULL, t);
       res[lane] = v;
+      const unsigned lead = __ballot_sync(SFMM_FULL, lane < nb && lane == __ffs(same) - 1);
+      if (lead >> lane & 1u) {
+        const int g = __popc(lead & lt);
+        s_gm[warp][g] = same;
+        s_gt[warp][g] = (unsigned char)t;
+      }
       __syncwarp();
-      if (lane < nb && lane == __ffs(same) - 1) {
-        unsigned m = same & (same - 1);
+      const double* const rd = reinterpret_cast<const double*>(res) + (lane & 3);
+      for (int g = lane >> 2; g < __popc(lead); g += 8) {
+        unsigned m = s_gm[warp][g];
+        double w = rd[4 * (__ffs(m) - 1)];
+        m &= m - 1;
         while (m) {
-          const double4_16a w = res[__ffs(m) - 1];
+          w += rd[4 * (__ffs(m) - 1)];
           m &= m - 1;
-          v.x += w.x;
-          v.y += w.y;
-          v.z += w.z;
-          v.w += w.w;
         }
-        double* const A = s_acc[warp][t];
-        A[0] += v.x;
-        A[1] += v.y;
-        A[2] += v.z;
-        A[3] += v.w;
+        s_acc[warp][s_gt[warp][g]][lane & 3] += w;
       }
       __syncwarp();
     };
