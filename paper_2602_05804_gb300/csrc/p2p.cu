@@ -3,12 +3,13 @@
 // combined with the far field, written in caller order (the momentum and
 // energy sums over the results are formed in reduce.cu).
 //
-// One warp per target leaf.  With n_t targets, lane l serves target
-// l mod n_t and takes every (32 / n_t)-th source ("phase" l / n_t), so that
-// all lanes work for any leaf size; sources are staged per warp in shared
-// memory, converted once to coordinates relative to the target leaf's
-// centre (FP32 form).
+// One warp per target leaf (or chunk of a long list).  With n_t targets, lane
+// l serves target l mod n_t and takes every (32 / n_t)-th source ("phase"
+// l / n_t), so that all lanes work for any leaf size; sources are staged per
+// warp in shared memory.  FP32 form: p2p_f32.cuh; FP64 form: p2p_fexp.cuh,
+// and k_p2p_fp64 below for what that leaves.
 #include <algorithm>
+#include <cfloat>
 #include <type_traits>
 
 #include "fexp.cuh"
@@ -19,6 +20,8 @@ namespace sfmm {
 #define P2P_WARPS 8
 #define P2P_NT (P2P_WARPS * 32)
 #define P2P_SB 128
+#define P64_WARPS 4  // the FP64 kernel's block
+#define P64_NT (P64_WARPS * 32)
 
 struct P2PArgs {
   const uint32_t* counts;  // the build's node and leaf counts (device)
@@ -98,26 +101,26 @@ __device__ __forceinline__ void m4_kernel(R q, R hinv, R ri, R& g, R& phi) {
   phi = out2 ? -ri : pk;
 }
 
-__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
-
-template <typename R> struct Vec4;
-template <> struct Vec4<float> { using T = float4; using T2 = float2; };
-template <> struct Vec4<double> { using T = double4_16a; using T2 = double2; };
-
 // Unsoftened pair: a -= m r^-3 d, phi -= m / r.
-template <typename R>
-__device__ __forceinline__ void pair_far(R xi, R yi, R zi, const typename Vec4<R>::T& s, R& ax, R& ay, R& az,
-                                         R& pt) {
-  const R dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
-  const R r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  const R ri = rsq(r2);
-  const R mr = s.w * ri;
-  const R mr3 = mr * (ri * ri);
+__device__ __forceinline__ void pair_far(double xi, double yi, double zi, const double4_16a& s, double& ax, double& ay,
+                                         double& az, double& pt) {
+  const double dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
+  const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+  const double ri = rsqrt(r2);
+  const double mr = s.w * ri;
+  const double mr3 = mr * (ri * ri);
   ax = fma(-mr3, dx, ax);
   ay = fma(-mr3, dy, ay);
   az = fma(-mr3, dz, az);
   pt -= mr;
+}
+
+// 1 / sqrt(x) of a normal number or infinity: one instruction (the library's
+// adds three that scale subnormal arguments).
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // Two unsoftened pairs of one target in the packed FP32 instructions (two
@@ -127,7 +130,7 @@ __device__ __forceinline__ void pair_far2(float2 xi, float2 yi, float2 zi, float
                                           float2 nm, float2& ax, float2& ay, float2& az, float2& pt) {
   const float2 dx = __fadd2_rn(xi, nx), dy = __fadd2_rn(yi, ny), dz = __fadd2_rn(zi, nz);
   const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-  const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+  const float2 ri = make_float2(rsqrt_normal(r2.x), rsqrt_normal(r2.y));
   const float2 mr = __fmul2_rn(nm, ri);                     // -m / r
   const float2 mr3 = __fmul2_rn(mr, __fmul2_rn(ri, ri));    // -m / r^3
   ax = __ffma2_rn(mr3, dx, ax);
@@ -138,34 +141,31 @@ __device__ __forceinline__ void pair_far2(float2 xi, float2 yi, float2 zi, float
 
 // Candidate pair: softened when r < 2 max(h_i, h_j) (mean of both kernels),
 // unsoftened otherwise; the self pair contributes nothing.
-template <typename R>
-__device__ __forceinline__ void pair_cand(R xi, R yi, R zi, R hinvi, R h2i, bool self,
-                                          const typename Vec4<R>::T& s, const typename Vec4<R>::T2& hh, R& ax,
-                                          R& ay, R& az, R& pt) {
-  const R dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
-  const R r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  const R ri = (r2 > R(0)) ? rsq(r2) : R(0);
-  R g, phi;
+__device__ __forceinline__ void pair_cand(double xi, double yi, double zi, double hinvi, double h2i, bool self,
+                                          const double4_16a& s, const double2& hh, double& ax,
+                                          double& ay, double& az, double& pt) {
+  const double dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
+  const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+  const double ri = (r2 > 0.0) ? rsqrt(r2) : 0.0;
+  double g, phi;
   if (r2 < fmax(h2i, hh.y)) {
-    const R r = r2 * ri;
-    R gi, pi, gj, pj;
-    m4_kernel<R>(r * hinvi, hinvi, ri, gi, pi);
-    m4_kernel<R>(r * hh.x, hh.x, ri, gj, pj);
-    g = R(0.5) * (gi + gj);
-    phi = R(0.5) * (pi + pj);
+    const double r = r2 * ri;
+    double gi, pi, gj, pj;
+    m4_kernel<double>(r * hinvi, hinvi, ri, gi, pi);
+    m4_kernel<double>(r * hh.x, hh.x, ri, gj, pj);
+    g = 0.5 * (gi + gj);
+    phi = 0.5 * (pi + pj);
   } else {
     g = ri * ri * ri;
     phi = -ri;
   }
-  const R m = self ? R(0) : s.w;
-  const R mg = m * g;
+  const double m = self ? 0.0 : s.w;
+  const double mg = m * g;
   ax = fma(-mg, dx, ax);
   ay = fma(-mg, dy, ay);
   az = fma(-mg, dz, az);
   pt = fma(m, phi, pt);
 }
-
-template <bool F32> __host__ __device__ constexpr int p2p_warps() { return F32 ? P2P_WARPS : P2P_WARPS / 2; }
 
 // Near sums v (a, Phi) of sorted particle i plus its far field: scaled by G
 // and written in caller order.
@@ -192,38 +192,39 @@ __device__ __forceinline__ void p2p_finish(const P2PArgs& a, int i, const R (&v)
 
 #include "p2p_fexp.cuh"
 
-// One warp per target leaf.  Sources: the particles of the leaf's neighbour
-// list, streamed 32 at a time over consecutive list entries (every lane
-// busy), moved to the target leaf's frame (FP32 form) and split once per
-// source into those that may lie inside the kernel of some target
-// (|x_j - s_L| < l_L + 2 max(h_max,L, h_j), with a small safety factor) and
-// those that cannot; the latter take the unsoftened branch-free loop.
-template <bool F32>
-__global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
-  using R = typename std::conditional<F32, float, double>::type;
-  using V = typename Vec4<R>::T;
-  using V2 = typename Vec4<R>::T2;
-  constexpr int NW = p2p_warps<F32>();
+#include "p2p_f32.cuh"
+
+// FP64 form, every step in FP64: the work items k_p2p_fexp leaves (values
+// outside its range).  Sources: the particles of the leaf's neighbour list,
+// streamed 32 at a time over consecutive list entries (every lane busy) and
+// split once per source into those that may lie inside the kernel of some
+// target (|x_j - s_L| < l_L + 2 max(h_max,L, h_j), with a small safety factor)
+// and those that cannot; the latter take the unsoftened branch-free loop.
+__global__ void __launch_bounds__(P64_NT, 1) k_p2p_fp64(const P2PArgs a) {
+  using R = double;
+  using V = double4_16a;
+  using V2 = double2;
+  constexpr int NW = P64_WARPS;
   constexpr int SB = P2P_SB;
   __shared__ V s_far[NW][SB];
   __shared__ V s_near[NW][SB];
   __shared__ V2 s_nhh[NW][SB];
   __shared__ short s_nloc[NW][SB];  // candidate's index in the target leaf, -1 outside it
-  __shared__ unsigned short s_sq[NW][F32 ? 1 : 64];  // FP64 softened pairs: candidate slot << 5 | owner lane
+  __shared__ unsigned short s_sq[NW][64];  // FP64 softened pairs: candidate slot << 5 | owner lane
   // phase sums at the end of a leaf; the FP64 softened-pair results during its loop
   __shared__ __align__(4 * sizeof(R)) R s_red[NW][4][32];
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = lanemask_lt();
   const int nextra = (int)a.d_split[0];
-  const int nitems = F32 ? nextra + (int)a.counts[1] : a.items[-4];
+  const int nitems = a.items[-4];
   unsigned long long pairs = 0;  // this lane's share of the pair evaluations
   while (true) {
     int item = 0;
     if (lane == 0) item = atomicAdd(a.leaf_counter, 1);
     item = __shfl_sync(SFMM_FULL, item, 0);
     if (item >= nitems) break;
-    if constexpr (!F32) item = a.items[item];
+    item = a.items[item];
     int leaf, chunk = 0;
     if (item < nextra) {
       const int2 x = a.extra[item];
@@ -237,7 +238,7 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
     const int fL = a.nfirst[L], nL = a.ncount[L];
     const float4 hiL = a.geo_hi[L], loL = a.geo_lo[L];
     const R lL = (R)hiL.w * R(1.0001), hL = (R)loL.w * R(1.0001);
-    const double cLx = F32 ? 0.0 : a.ncx[L], cLy = F32 ? 0.0 : a.ncy[L], cLz = F32 ? 0.0 : a.ncz[L];
+    const double cLx = a.ncx[L], cLy = a.ncy[L], cLz = a.ncz[L];
     // lane -> (target slot, phase)
     const int nph = (nL <= 16) ? (32 / nL) : 1;
     const int ntl = (nL <= 32) ? nL : 32;
@@ -250,14 +251,8 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
     R xi0 = R(0), yi0 = R(0), zi0 = R(0), hinvi0 = R(0), h2i0 = R(0);
     R xi1 = R(0), yi1 = R(0), zi1 = R(0), hinvi1 = R(0), h2i1 = R(0);
     auto load_target = [&](int i, R& x, R& y, R& z, R& hinv, R& h2) {
-      if constexpr (F32) {
-        const float4 p = a.prel[i];
-        const float4 hh = a.phh[i];
-        x = p.x; y = p.y; z = p.z; hinv = hh.x; h2 = hh.y;
-      } else {
-        const double h = a.ph[i];
-        x = a.px[i]; y = a.py[i]; z = a.pz[i]; hinv = 1.0 / h; h2 = 4.0 * h * h;
-      }
+      const double h = a.ph[i];
+      x = a.px[i]; y = a.py[i]; z = a.pz[i]; hinv = 1.0 / h; h2 = 4.0 * h * h;
     };
     if (on0) load_target(fL + t0, xi0, yi0, zi0, hinvi0, h2i0);
     if (on1) load_target(fL + t1, xi1, yi1, zi1, hinvi1, h2i1);
@@ -275,7 +270,6 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
     int e = 0;                 // next list entry to load
     int tot = 0, pdone = 0;    // particles of the loaded entries / staged so far
     int cum = 0, fS = 0;       // this lane's entry: first particle in the stream, first particle index
-    R ox = R(0), oy = R(0), oz = R(0);
     while (true) {
       const bool stream_left = (pdone < tot) || (e < cnt);
       if (stream_left && pdone == tot) {
@@ -287,12 +281,6 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
           fS = a.nfirst[S];
           nS = a.ncount[S];
           pairs += (unsigned long long)nL * nS - (S == L ? nL : 0);
-          if constexpr (F32) {
-            const float4 hS = a.geo_hi[S], lS = a.geo_lo[S];
-            ox = df_diff(hS.x, lS.x, hiL.x, loL.x);
-            oy = df_diff(hS.y, lS.y, hiL.y, loL.y);
-            oz = df_diff(hS.z, lS.z, hiL.z, loL.z);
-          }
         }
         int incl = nS;
 #pragma unroll
@@ -318,36 +306,21 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
         const int before = __popc(__ballot_sync(SFMM_FULL, pre));
         const int l = before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
         const int d_l = __shfl_sync(SFMM_FULL, fS - cum, l);  // particle index minus stream position
-        const R ox_l = __shfl_sync(SFMM_FULL, ox, l), oy_l = __shfl_sync(SFMM_FULL, oy, l),
-                oz_l = __shfl_sync(SFMM_FULL, oz, l);
         V v;
         V2 hh;
-        R h2j = R(0);  // 2 h_j (FP32 form: rounded up)
+        R h2j = R(0);  // 2 h_j
         int i = 0;
         if (valid) {
           i = d_l + p;
-          if constexpr (F32) {
-            const float4 q = a.prel[i];
-            v = make_float4(q.x + ox_l, q.y + oy_l, q.z + oz_l, q.w);
-            const float4 hr = a.phh[i];
-            hh = make_float2(hr.x, hr.y);
-            h2j = hr.z;
-          } else {
-            const double h = a.ph[i];
-            v = make_double4_16a(a.px[i], a.py[i], a.pz[i], a.pm[i]);
-            hh = make_double2(1.0 / h, 4.0 * h * h);
-            h2j = 2.0 * h;
-          }
+          const double h = a.ph[i];
+          v = make_double4_16a(a.px[i], a.py[i], a.pz[i], a.pm[i]);
+          hh = make_double2(1.0 / h, 4.0 * h * h);
+          h2j = 2.0 * h;
         } else {
           v.x = v.y = v.z = v.w = R(0);
           hh.x = hh.y = R(0);
         }
-        R rx = v.x, ry = v.y, rz = v.z;
-        if constexpr (!F32) {
-          rx -= cLx;
-          ry -= cLy;
-          rz -= cLz;
-        }
+        const R rx = v.x - cLx, ry = v.y - cLy, rz = v.z - cLz;
         // reach = l_L + 2 max(h_L, h_j) (l_L and h_L carry a 1.0001 margin)
         const R reach = lL + fmax(R(2) * hL, h2j);
         const bool near = valid && (fma(rx, rx, fma(ry, ry, rz * rz)) < reach * reach);
@@ -359,18 +332,7 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
           s_nloc[warp][q] = (short)((i >= fL && i < fL + nL) ? i - fL : -1);
         } else if (valid) {
           const int q = nfar + __popc(bf & lt);
-          if constexpr (F32) {
-            // pairs of sources, negated: {x0, x1, y0, y1}, {z0, z1, m0, m1}
-            float* const fxy = reinterpret_cast<float*>(&s_far[warp][q >> 1]);
-            float* const fzm = reinterpret_cast<float*>(&s_far[warp][SB / 2 + (q >> 1)]);
-            const int hb = q & 1;
-            fxy[hb] = -v.x;
-            fxy[2 + hb] = -v.y;
-            fzm[hb] = -v.z;
-            fzm[2 + hb] = -v.w;
-          } else {
-            s_far[warp][q] = v;
-          }
+          s_far[warp][q] = v;
         }
         nnear += __popc(bn);
         nfar += __popc(bf);
@@ -379,73 +341,33 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
       const bool last = !((pdone < tot) || (e < cnt));
       if (!(nfar > SB - 32 || nnear > SB - 32 || last)) continue;
       __syncwarp();
-      if constexpr (F32) {
-        if (nfar & 1) {
-          // odd count: the last pair's second source repeats the first with
-          // no mass (outside every kernel, so r > 0)
-          if (lane == 0) {
-            float* const fxy = reinterpret_cast<float*>(&s_far[warp][nfar >> 1]);
-            float* const fzm = reinterpret_cast<float*>(&s_far[warp][SB / 2 + (nfar >> 1)]);
-            fxy[1] = fxy[0];
-            fxy[3] = fxy[2];
-            fzm[1] = fzm[0];
-            fzm[3] = 0.0f;
-          }
-          __syncwarp();
-        }
-      }
-      if (lane_on) {
+      if (nL > 32) {
         // unsoftened sources
-        if constexpr (F32) {
-          // one pass per target slot (the second only for leaves of more
-          // than 32 particles)
-          const int np = (nfar + 1) >> 1;
-          auto far_pass = [&](float xi, float yi, float zi, float& ax, float& ay, float& az, float& pt) {
-            const float2 x2 = make_float2(xi, xi), y2 = make_float2(yi, yi), z2 = make_float2(zi, zi);
-            float2 fx = make_float2(0.0f, 0.0f), fy = fx, fz = fx, fp = fx;
-            for (int pj = ph; pj < np; pj += nph) {
-              const float4 a = s_far[warp][pj], b = s_far[warp][SB / 2 + pj];
-              pair_far2(x2, y2, z2, make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
-                        make_float2(b.z, b.w), fx, fy, fz, fp);
-            }
-            ax += fx.x + fx.y;
-            ay += fy.x + fy.y;
-            az += fz.x + fz.y;
-            pt += fp.x + fp.y;
-          };
-          far_pass(xi0, yi0, zi0, ax0, ay0, az0, pt0);
-          if (nL > 32) far_pass(xi1, yi1, zi1, ax1, ay1, az1, pt1);
-        } else if (nL > 32) {
-        // FP64 form, more than 32 targets (up to 32: balanced, below)
+        // more than 32 targets (up to 32: balanced, below)
         int j = ph;
         for (; j + nph < nfar; j += 2 * nph) {
           const V s0 = s_far[warp][j], s1 = s_far[warp][j + nph];
-          pair_far<R>(xi0, yi0, zi0, s0, ax0, ay0, az0, pt0);
-          pair_far<R>(xi0, yi0, zi0, s1, ax0, ay0, az0, pt0);
-          if (nL > 32) {
-            pair_far<R>(xi1, yi1, zi1, s0, ax1, ay1, az1, pt1);
-            pair_far<R>(xi1, yi1, zi1, s1, ax1, ay1, az1, pt1);
-          }
+          pair_far(xi0, yi0, zi0, s0, ax0, ay0, az0, pt0);
+          pair_far(xi0, yi0, zi0, s1, ax0, ay0, az0, pt0);
+          pair_far(xi1, yi1, zi1, s0, ax1, ay1, az1, pt1);
+          pair_far(xi1, yi1, zi1, s1, ax1, ay1, az1, pt1);
         }
         if (j < nfar) {
           const V s0 = s_far[warp][j];
-          pair_far<R>(xi0, yi0, zi0, s0, ax0, ay0, az0, pt0);
-          if (nL > 32) pair_far<R>(xi1, yi1, zi1, s0, ax1, ay1, az1, pt1);
-        }
+          pair_far(xi0, yi0, zi0, s0, ax0, ay0, az0, pt0);
+          pair_far(xi1, yi1, zi1, s0, ax1, ay1, az1, pt1);
         }
         // candidates inside some kernel of the leaf, softened in place
-        if (F32 || nL > 32) {
-          for (int jn = ph; jn < nnear; jn += nph) {
-            const V s0 = s_near[warp][jn];
-            const V2 hh = s_nhh[warp][jn];
-            const int loc = s_nloc[warp][jn];
-            pair_cand<R>(xi0, yi0, zi0, hinvi0, h2i0, loc == t0, s0, hh, ax0, ay0, az0, pt0);
-            if (nL > 32) pair_cand<R>(xi1, yi1, zi1, hinvi1, h2i1, loc == t1, s0, hh, ax1, ay1, az1, pt1);
-          }
+        for (int jn = ph; jn < nnear; jn += nph) {
+          const V s0 = s_near[warp][jn];
+          const V2 hh = s_nhh[warp][jn];
+          const int loc = s_nloc[warp][jn];
+          pair_cand(xi0, yi0, zi0, hinvi0, h2i0, loc == t0, s0, hh, ax0, ay0, az0, pt0);
+          pair_cand(xi1, yi1, zi1, hinvi1, h2i1, loc == t1, s0, hh, ax1, ay1, az1, pt1);
         }
       }
-      if (!F32 && nL <= 32 && nfar > 0) {
-        // FP64 form, up to 32 targets: the nL x nfar unsoftened pairs (target
+      if (nL <= 32 && nfar > 0) {
+        // up to 32 targets: the nL x nfar unsoftened pairs (target
         // major) cut into 32 equal runs, one per lane -- every lane busy, and
         // FP64 work costs per warp instruction whatever the active lanes.  A
         // run spans at most two targets; the partials go back to the lane
@@ -470,7 +392,7 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
               y = a.py[fL + t];
               z = a.pz[fL + t];
             }
-            pair_far<R>(x, y, z, s_far[warp][j], fx, fy, fz, fp);
+            pair_far(x, y, z, s_far[warp][j], fx, fy, fz, fp);
             ++j;
           }
         }
@@ -517,15 +439,14 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
         }
         __syncwarp();
       }
-      if (!F32 && nL <= 32 && nnear > 0) {
-        // FP64 form, up to 32 targets: the unsoftened candidates in place; a
+      if (nL <= 32 && nnear > 0) {
+        // up to 32 targets: the unsoftened candidates in place; a
         // pair inside a kernel goes to the warp's queue, and every 32 queued
         // pairs are evaluated one per lane (target records by shuffle from the
         // lane holding them) and handed back to their owner lanes, which add
         // them in queue order.  The FP64 pipe costs the same per warp
         // instruction whatever the active lanes, so the softened branch pays
-        // only once per 32 pairs; in the FP32 form the in-place branch is
-        // faster (measured)
+        // only once per 32 pairs
         V* const s_soft = reinterpret_cast<V*>(&s_red[warp][0][0]);
         auto soft_batch = [&](int cnt, unsigned mine) {
           __syncwarp();
@@ -541,11 +462,11 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
             const V2 hh = s_nhh[warp][jn];
             const R dx = tx - s0.x, dy = ty - s0.y, dz = tz - s0.z;
             const R r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            const R ri = (r2 > R(0)) ? rsq(r2) : R(0);
+            const R ri = (r2 > R(0)) ? rsqrt(r2) : R(0);
             const R r = r2 * ri;
             R gi, pi, gj, pj;
-            m4_kernel<R>(r * thinv, thinv, ri, gi, pi);
-            m4_kernel<R>(r * hh.x, hh.x, ri, gj, pj);
+            m4_kernel<double>(r * thinv, thinv, ri, gi, pi);
+            m4_kernel<double>(r * hh.x, hh.x, ri, gj, pj);
             const R mg = s0.w * (R(0.5) * (gi + gj));
             c.x = -mg * dx;
             c.y = -mg * dy;
@@ -579,7 +500,7 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
             ins = !self && r2 < fmax(h2i0, hh.y);
             // outside both kernels: unsoftened (r >= 2 h > 0); else nothing here
             const bool skip = self || ins;
-            const R ri = rsq(skip ? R(1) : r2);
+            const R ri = rsqrt(skip ? R(1) : r2);
             const R mr = (skip ? R(0) : s0.w) * ri;
             const R mr3 = mr * (ri * ri);
             ax0 = fma(-mr3, dx, ax0);
@@ -637,7 +558,7 @@ __global__ void __launch_bounds__(P2P_NT, F32 ? 3 : 1) k_p2p(const P2PArgs a) {
           v[c] = sacc;
         }
         if (pslot < 0) {
-          p2p_finish<F32>(a, fL + t, v);
+          p2p_finish<false>(a, fL + t, v);
         } else {
           R* pp = static_cast<R*>(a.part) + ((size_t)(pslot + chunk) * a.lmax + t) * 4;
 #pragma unroll
@@ -714,11 +635,14 @@ __global__ void k_p2p_combine(const P2PArgs a) {
 }
 
 int p2p_blocks_fit(sfmm_ctx* c) {
-  const bool f32 = (c->precision == SFMM_FP32);
-  const int nt = 32 * p2p_warps<true>();
   int per_sm = 0;
-  if (f32) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p<true>, nt, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_fexp, FX_NT, 0);
+  if (c->precision == SFMM_FP32) {
+    const int smem = P2P_WARPS * (int)sizeof(P2PWarp);
+    cudaFuncSetAttribute(k_p2p_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_f32, P2P_NT, smem);
+  } else {
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_fexp, FX_NT, 0);
+  }
   return per_sm < 1 ? 1 : per_sm;
 }
 
@@ -736,11 +660,10 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   SFMM_CUDA_TRY(cudaMemsetAsync(ctr + 10, 0, 4 * sizeof(unsigned long long), c->stream));
   const bool f32 = (c->precision == SFMM_FP32);
   // the grids: one block per resident slot
-  const int nt = 32 * (f32 ? p2p_warps<true>() : p2p_warps<false>());
   const int fit = p2p_blocks_fit(c);
   const int per_sm = (c->p2p_blocks > 0 && c->p2p_blocks < fit) ? c->p2p_blocks : fit;  // option: fewer
   const int nblocks = per_sm * num_sms(c->device);
-  const int want = 8 * nblocks * (f32 ? p2p_warps<true>() : FX_WARPS);
+  const int want = 8 * nblocks * (f32 ? P2P_WARPS : FX_WARPS);
   // long lists: slots, extra items and split leaves are counted by the split
   // pass on the device; the buffers are sized from bounds on the host (a list
   // of cnt > chunk entries takes ceil(cnt / chunk) <= 2 cnt / chunk slots, and
@@ -803,7 +726,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   a.chunk_now = ctr + 7;
   a.pair_counter = ctr + 3;
   if (f32) {
-    k_p2p<true><<<nblocks, nt, 0, c->stream>>>(a);
+    k_p2p_f32<<<nblocks, P2P_NT, P2P_WARPS * sizeof(P2PWarp), c->stream>>>(a);
   } else {
     // FP32-pipe expansions first; what they cannot take (usually nothing)
     // is left to the FP64 kernel
@@ -827,7 +750,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
     k_p2p_fexp<<<nblocks, FX_NT, 0, c->stream>>>(a, f);
     a.leaf_counter = f.fb + 1;
     a.items = f.fb + 4;
-    k_p2p<false><<<num_sms(c->device), nt, 0, c->stream>>>(a);
+    k_p2p_fp64<<<num_sms(c->device), P64_NT, 0, c->stream>>>(a);
     c->nlaunch += 2;
   }
   ++c->nlaunch;

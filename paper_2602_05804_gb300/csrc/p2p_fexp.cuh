@@ -11,7 +11,7 @@
 // three floats (exactly for |x| >= 2^-18, else to 2^-71), masses scaled by a
 // power of two to below the total and split likewise, (2h)^2 rounded up.
 // A leaf whose smallest 2h is below 2^-18 of that scale, a source mass below
-// 2^-80 of the total, or a scale outside 2^+-300 go to k_p2p<false>: its
+// 2^-80 of the total, or a scale outside 2^+-300 go to k_p2p_fp64: its
 // FP64 arithmetic has no such limits.
 
 // Powers of two of a system: positions by 2^-kx, masses by 2^-km.
@@ -30,7 +30,7 @@ struct FexpArgs {
   float4* rec2;         // {x, y, z (rest), m (rest)}
   float2* rech;         // {(2h)^2 rounded up, 2h rounded down}, scaled
   double2* hinv;        // {1 / h, 1 / h^3}
-  int* fb;              // [0] work items left to k_p2p<false>, [1] its item counter, [4 ..] the items
+  int* fb;              // [0] work items left to k_p2p_fp64, [1] its item counter, [4 ..] the items
 };
 
 __device__ __forceinline__ SysScale sys_scale(const P2PArgs& a, const FexpArgs& f, int sorted) {
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256) k_fexp_records(const P2PArgs a, const Fex
     const double hi = 1.0 / a.ph[i];
     f.hinv[i] = make_double2(hi, hi * hi * hi);
     const SysScale s = sys_scale(a, f, i);
-    if (!s.ok) continue;  // (not read: every leaf of the system goes to k_p2p<false>)
+    if (!s.ok) continue;  // (not read: every leaf of the system goes to k_p2p_fp64)
     const double sx = __hiloint2double((1023 - s.kx) << 20, 0), sm = __hiloint2double((1023 - s.km) << 20, 0);
     float4 r0, r1, r2;
     fexp::split_grid(a.px[i] * sx, r0.x, r1.x, r2.x);

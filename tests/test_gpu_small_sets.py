@@ -1,0 +1,64 @@
+"""Paths that small sets and batches take: the one-block sort and scan at the
+edges of their ranges (4096 particles, 8192 values), sums over slices of 8192
+particles of a system, and neighbour lists cut finer than the option when the
+lists are few."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from gpu_helpers import TOL_FP64, acc_rel, pot_rel, solver
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 1023, 1024, 1025, 2049, 4095, 4096, 4097, 8191, 8192, 8193])
+def test_sorted_order_and_tree(n):
+    pos, m, h = workloads.plummer(n, 300 + n)
+    pos[n // 3:n // 2] = pos[n // 3]  # equal keys: input order decides
+    s = solver("fp32")
+    s.build(pos, m, h, 8)
+    t = s.tree()
+    s.close()
+    o = oracle.Tree(pos, m, h, 8, p=0)
+    assert np.array_equal(t["perm"], o.perm)
+    for k in ("first", "count", "right"):
+        assert np.array_equal(t[k], getattr(o, k)), k
+
+
+def test_sums_of_sliced_systems():
+    sizes = [1, 8191, 8192, 8193, 20001]
+    parts = [workloads.plummer(k, 50 + k) for k in sizes]
+    pos, m, h = (np.concatenate([p[q] for p in parts]) for q in range(3))
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    s = solver("fp64")
+    s.build_batch(off, pos, m, h, np.full(len(sizes), 8, np.int32))
+    acc, pot = (t.cpu().numpy() for t in s.gravity(0.7, 1))
+    sums, st = s.batch_sums(), s.stats()
+    s.close()
+    ma = m[:, None] * acc
+    for k, (a, b) in enumerate(zip(off[:-1], off[1:])):
+        for c in range(3):
+            x = ma[a:b, c]
+            assert abs(sums[k, c] - math.fsum(x)) <= 4e-16 * abs(math.fsum(x)) + 1e-25 * np.abs(x).sum()
+        assert abs(sums[k, 3] - math.fsum(np.abs(ma[a:b]).ravel())) <= 1e-14 * sums[k, 3]
+        assert abs(sums[k, 4] - 0.5 * math.fsum(m[a:b] * pot[a:b])) <= 1e-14 * abs(sums[k, 4])
+    for c in range(3):
+        assert abs(st["momentum"][c] - math.fsum(ma[:, c])) <= 4e-16 * abs(math.fsum(ma[:, c])) + 1e-25 * np.abs(ma).sum()
+    assert abs(st["W"] - 0.5 * math.fsum(m * pot)) <= 1e-14 * abs(st["W"])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("n,leaf", [(60, 4), (700, 16), (700, 64), (5000, 33)])
+def test_few_lists_are_cut_finer(prec, n, leaf):
+    pos, m, h = workloads.binary_polytrope(n, 9)
+    a_o, p_o, _ = oracle.sfmm(pos, m, h, theta=0.4, p=2, leaf_size=leaf)
+    tol = TOL_FP64 if prec == "fp64" else 3e-5
+    for chunk in (32, 65536):
+        s = solver(prec, p2p_chunk=chunk)
+        s.build(pos, m, h, leaf)
+        acc, pot = (t.cpu().numpy() for t in s.gravity(0.4, 2))
+        s.close()
+        assert acc_rel(acc, a_o).max() <= tol and pot_rel(pot, p_o).max() <= tol
