@@ -205,23 +205,23 @@ def gen_m2m(p):
 
 
 def gen_tables(p):
-    """Lane-parallel L2L: for target coefficient i and source j of the same
-    block (M or F) with gamma_j >= beta_i, index of h^(gamma_j - beta_i)/()!
-    in sfmm_mono_{p+1}; -1 otherwise."""
+    """Lane-parallel L2L: target coefficient j is its own source plus
+    h^(gamma_i - beta_j)/()! C_i over the other sources i of its block (M or F)
+    with gamma_i >= beta_j; step k of lane j holds i + 256 t, t the index of
+    the monomial in sfmm_mono_{p+1} (0xffff: no more terms)."""
     IM = mis(p)
     IF = mis(p + 1, 1)
     allc = [("M", g) for g in IM] + [("F", g) for g in IF]
     Imono = idx_of(p + 1)
     n = len(allc)
-    rows = []
-    for i, (bi, b) in enumerate(allc):
-        row = []
-        for j, (bj, g) in enumerate(allc):
-            row.append(Imono[sub(g, b)] if (bi == bj and geq(g, b)) else -1)
-        rows.append(row)
-    body = ",\n  ".join("{" + ", ".join("%d" % v for v in r) + "}" for r in rows)
+    rows = [[i + 256 * Imono[sub(g, b)] for i, (bi, g) in enumerate(allc) if bi == bj and g != b and geq(g, b)]
+            for bj, b in allc]
+    steps, stride = max(1, max(len(r) for r in rows)), (n + 31) // 32 * 32
+    body = ",\n  ".join("{" + ", ".join("%d" % (rows[j][k] if j < n and k < len(rows[j]) else 0xffff)
+                                         for j in range(stride)) + "}" for k in range(steps))
     mi_rows = ", ".join("{%d,%d,%d}" % g for g in IM)
-    return ("static __device__ const signed char sfmm_l2l_table_%d[%d][%d] = {\n  %s};\n" % (p, n, n, body)
+    return ("#define SFMM_NT_%d %d  /* steps of the L2L translation */\n" % (p, steps)
+            + "static __device__ const unsigned short sfmm_l2l_steps_%d[%d][%d] = {\n  %s};\n" % (p, steps, stride, body)
             + "static const int sfmm_moment_mi_%d[%d][3] = {%s};\n" % (p, len(IM), mi_rows))
 
 

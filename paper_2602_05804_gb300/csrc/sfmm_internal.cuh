@@ -68,7 +68,7 @@ struct sfmm_ctx {
   int walk_mode = 1;        // 1: per-node shared pairs (default), 0: per-leaf replay (Algorithm 1),
                             // 2: per-node pairs, each evaluated once for both sides
   int schedule = 0;         // walk mode 1: 0 automatic, 1 one launch per depth, 2 readiness queue
-  int p2p_chunk = SFMM_P2P_CHUNK_DEFAULT;  // neighbour-list entries per near-field work item
+  int p2p_chunk = SFMM_P2P_CHUNK_DEFAULT;  // most neighbour-list entries per near-field work item
   int p2p_blocks = 0;       // near-field blocks per SM (0: as many as fit)
   int max_depth = 0;
   std::vector<int> h_level_off;  // host copy: internal nodes per depth, max_depth + 2 entries
@@ -125,7 +125,6 @@ struct sfmm_ctx {
   const double* red_acc = nullptr;  // outputs of the last near-field pass (caller order), read by the sums
   const double* red_pot = nullptr;
   int64_t arena_used = 0;
-  int64_t split_chunks = 0, split_lists = 0;  // from the walk: chunks of split lists, split lists
   int64_t walk_arena_cap = 0, walk_cf_cap = 0;  // list and child-list capacities of the last walk
 
   // status word (device) + pinned host mirror

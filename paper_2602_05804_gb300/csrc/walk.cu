@@ -33,11 +33,11 @@ __global__ void __launch_bounds__(WALK_NT) k_walk(const WalkArgs a) {
   __shared__ int s_queue[WALK_WARPS][WALK_MQ];
   __shared__ R s_T[WALK_WARPS][NCS * 32];
   __shared__ R s_h[WALK_WARPS][E::NMONO1];
-  __shared__ signed char s_tab[NC * NC];
+  __shared__ unsigned short s_tab[E::NT * E::TS];
 
   if (COMPUTE) {
-    const signed char* tab = E::table();
-    for (int t = threadIdx.x; t < NC * NC; t += WALK_NT) s_tab[t] = tab[t];
+    const unsigned short* tab = E::table();
+    for (int t = threadIdx.x; t < E::NT * E::TS; t += WALK_NT) s_tab[t] = tab[t];
   }
   __syncthreads();
 
@@ -221,12 +221,7 @@ __global__ void __launch_bounds__(WALK_NT) k_walk(const WalkArgs a) {
           for (int b = 0; b < NCS; ++b) {
             const int j = lane + 32 * b;
             if (j < NC) {
-              R corr = R(0);
-              const signed char* row = s_tab + j * NC;
-              for (int i = 0; i < NC; ++i) {
-                const int t = row[i];
-                if (t > 0) corr = fma(s_h[warp][t], s_T[warp][i], corr);
-              }
+              const R corr = shift_sum<P>(j, s_h[warp], s_T[warp], s_tab);
               if constexpr (F32) {
                 dfloat r = df_add_f(dfloat{Tn[b], Tl[b]}, corr);
                 Tn[b] = r.hi;
@@ -330,10 +325,6 @@ __global__ void __launch_bounds__(WALK_NT) k_walk(const WalkArgs a) {
         a.p2p_off[leaf] = (long long)base;
         a.p2p_cnt[leaf] = nn;
         st_pl += nn;
-        if (nn > a.chunk) {
-          atomicAdd(a.split_counter, (unsigned long long)((nn + a.chunk - 1) / a.chunk));
-          atomicAdd(a.split_counter + 1, 1ull);
-        }
       }
     }
     __syncwarp();
@@ -430,8 +421,6 @@ int run_walk(sfmm_ctx* c, double theta, int order, bool dump, int64_t cap_m2l, i
     a.leaf_counter = reinterpret_cast<int*>(ctr + 8);
     a.arena = c->arena.as<int>();
     a.arena_counter = ctr + 9;
-    a.split_counter = ctr + 5;
-    a.chunk = c->p2p_chunk;
     a.arena_cap = arena_cap;
     a.p2p_off = c->p2p_off.as<long long>();
     a.p2p_cnt = c->p2p_cnt.as<int>();
@@ -474,8 +463,6 @@ int run_walk(sfmm_ctx* c, double theta, int order, bool dump, int64_t cap_m2l, i
     SFMM_CUDA_TRY(cudaMemcpy(c->h_scalars, ctr, sizeof(unsigned long long) * 10, cudaMemcpyDeviceToHost));
     const unsigned long long* hs = reinterpret_cast<const unsigned long long*>(c->h_scalars);
     c->arena_used = (int64_t)hs[9];
-    c->split_chunks = (int64_t)hs[5];
-    c->split_lists = (int64_t)hs[6];
     c->stats.m2l = (int64_t)hs[0];
     c->stats.m2l_unique = (int64_t)hs[1];
     c->stats.p2p_leaves = (int64_t)hs[2];
@@ -512,8 +499,6 @@ int run_walk_dump_write(sfmm_ctx* c, double theta, const long long* d_off, int* 
   a.leaf_counter = reinterpret_cast<int*>(ctr + 8);
   a.arena = c->arena.as<int>();
   a.arena_counter = ctr + 9;
-  a.split_counter = ctr + 5;
-    a.chunk = c->p2p_chunk;
   a.arena_cap = (long long)(c->arena.bytes / sizeof(int));
   a.p2p_off = c->p2p_off.as<long long>();
   a.p2p_cnt = c->p2p_cnt.as<int>();

@@ -44,8 +44,6 @@ struct WalkArgs {
   int* leaf_counter;
   int* arena;
   unsigned long long* arena_counter;
-  unsigned long long* split_counter;  // [0]: chunks of split lists, [1]: split lists
-  int chunk;                          // neighbour-list entries per near-field work item
   long long arena_cap;
   long long* p2p_off;
   int* p2p_cnt;
@@ -75,7 +73,8 @@ template <int P> struct Exp;
     template <typename T, typename U> __device__ static void l2p(const T* am, const U* C, T* o) { sfmm_l2p_##PP(am, C, o); } \
     template <typename T> __device__ static void mono(T x, T y, T z, T* o) { sfmm_mono_##PP(x, y, z, o); }     \
     template <typename T> __device__ static void mono1(T x, T y, T z, T* o) { sfmm_mono_##PP1(x, y, z, o); }   \
-    __device__ static const signed char* table() { return &sfmm_l2l_table_##PP[0][0]; }                       \
+    static constexpr int NT = SFMM_NT_##PP, TS = (NC + 31) / 32 * 32;  /* L2L: steps, stride */                \
+    __device__ static const unsigned short* table() { return &sfmm_l2l_steps_##PP[0][0]; }                    \
     /* independent components (at most one z): source rows, sums, their unfolding */                           \
     static constexpr int NR = SFMM_NR_##PP, NS = SFMM_NS_##PP, NX = SFMM_NX_##PP;                              \
     template <typename T> __device__ static void fold(const T* Q, T* q) { sfmm_fold_##PP(Q, q); }              \
@@ -108,6 +107,20 @@ template <int P>
 __device__ __forceinline__ void node_offset(const WalkArgs& a, int v, double (&d)[3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) d[c] = a.row64 ? a.row64[(size_t)v * row_len<P, false>() + 3 + c] : 0.0;
+}
+
+// Sum of the translated terms of coefficient j (App. A.2): h the monomials of
+// the shift, T the source coefficients.  9 steps at p = 2 and 34 at p = 4,
+// where a walk over every source took 29 and 90.
+template <int P, typename R>
+__device__ __forceinline__ R shift_sum(int j, const R* h, const R* T, const unsigned short* s_tab) {
+  R corr = R(0);
+#pragma unroll 9
+  for (int k = 0; k < Exp<P>::NT; ++k) {
+    const int e = s_tab[k * Exp<P>::TS + j];
+    if (e != 0xffff) corr = fma(h[e >> 8], T[e & 255], corr);
+  }
+  return corr;
 }
 
 // Reduce-scatter over the warp: on entry every lane holds v[0..32); on exit

@@ -107,11 +107,12 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? 4 : 1) k_walk_pair(
   __shared__ int s_queue[WALK_WARPS][2][WALK_MQ];
   __shared__ R s_T[WALK_WARPS][NCS * 32];
   __shared__ R s_h[WALK_WARPS][E::NMONO1];
-  __shared__ signed char s_tab[NC * NC];
+  __shared__ unsigned short s_tab[E::NT * E::TS];
   __shared__ signed char s_unf[NC * 2 * E::NX];
   {
-    const signed char *tab = E::table(), *unf = E::unfold();
-    for (int t = threadIdx.x; t < NC * NC; t += WALK_NT) s_tab[t] = tab[t];
+    const unsigned short* tab = E::table();
+    const signed char* unf = E::unfold();
+    for (int t = threadIdx.x; t < E::NT * E::TS; t += WALK_NT) s_tab[t] = tab[t];
     for (int t = threadIdx.x; t < NC * 2 * E::NX; t += WALK_NT) s_unf[t] = unf[t];
   }
   __syncthreads();
@@ -374,10 +375,6 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? 4 : 1) k_walk_pair(
           a.p2p_off[leaf] = (long long)base;
           a.p2p_cnt[leaf] = nn;
           st_pl += nn;
-          if (nn > a.chunk) {
-            atomicAdd(a.split_counter, (unsigned long long)((nn + a.chunk - 1) / a.chunk));
-            atomicAdd(a.split_counter + 1, 1ull);
-          }
         }
       }
       __syncwarp();

@@ -82,7 +82,7 @@ __device__ __forceinline__ void node_coefficients(const LevelArgs& la, int A, in
                                                   typename std::conditional<F32, float, double>::type* Tn,
                                                   float* Tl, typename std::conditional<F32, float, double>::type* sT,
                                                   typename std::conditional<F32, float, double>::type* sH,
-                                                  const signed char* s_tab, int lane) {
+                                                  const unsigned short* s_tab, int lane) {
   using E = Exp<P>;
   using R = typename std::conditional<F32, float, double>::type;
   constexpr int NC = E::NC;
@@ -130,12 +130,7 @@ __device__ __forceinline__ void node_coefficients(const LevelArgs& la, int A, in
     for (int b = 0; b < NCS; ++b) {
       const int j = lane + 32 * b;
       if (j < NC) {
-        R corr = R(0);
-        const signed char* row = s_tab + j * NC;
-        for (int i = 0; i < NC; ++i) {
-          const int t = row[i];
-          if (t > 0) corr = fma(sH[t], sT[i], corr);
-        }
+        const R corr = shift_sum<P>(j, sH, sT, s_tab);
         if constexpr (F32) {
           dfloat r = df_add_f(dfloat{Tn[b], Tl[b]}, corr);
           Tn[b] = r.hi;
@@ -229,11 +224,11 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
   __shared__ float4 s_qr[WALK_WARPS][F32 ? WALK_MQ : 1];  // accepted pairs' separation s_B - s_A
   __shared__ R s_T[WALK_WARPS][NCS * 32];
   __shared__ R s_h[WALK_WARPS][E::NMONO1];
-  __shared__ signed char s_tab[NC * NC];
+  __shared__ unsigned short s_tab[E::NT * E::TS];
   __shared__ signed char s_unf[SYM ? 1 : NC * 2 * E::NX];
   {
-    const signed char* tab = E::table();
-    for (int t = threadIdx.x; t < NC * NC; t += WALK_NT) s_tab[t] = tab[t];
+    const unsigned short* tab = E::table();
+    for (int t = threadIdx.x; t < E::NT * E::TS; t += WALK_NT) s_tab[t] = tab[t];
     if constexpr (!SYM) {
       const signed char* unf = E::unfold();
       for (int t = threadIdx.x; t < NC * 2 * E::NX; t += WALK_NT) s_unf[t] = unf[t];
@@ -575,10 +570,6 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
         a.p2p_off[leaf] = (long long)base;
         a.p2p_cnt[leaf] = nn;
         st_pl += nn;
-        if (nn > a.chunk) {
-          atomicAdd(a.split_counter, (unsigned long long)((nn + a.chunk - 1) / a.chunk));
-          atomicAdd(a.split_counter + 1, 1ull);
-        }
       }
     }
     __syncwarp();
@@ -611,10 +602,10 @@ __global__ void __launch_bounds__(WALK_NT) k_walk_finalize(const LevelArgs la, i
   const WalkArgs& a = la.w;
   __shared__ R s_T[WALK_WARPS][NCS * 32];
   __shared__ R s_h[WALK_WARPS][E::NMONO1];
-  __shared__ signed char s_tab[NC * NC];
+  __shared__ unsigned short s_tab[E::NT * E::TS];
   {
-    const signed char* tab = E::table();
-    for (int t = threadIdx.x; t < NC * NC; t += WALK_NT) s_tab[t] = tab[t];
+    const unsigned short* tab = E::table();
+    for (int t = threadIdx.x; t < E::NT * E::TS; t += WALK_NT) s_tab[t] = tab[t];
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -826,8 +817,6 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
     a.ring_cap = c->ring_capacity;
     a.arena = c->arena.as<int>();
     a.arena_counter = ctr + 9;
-    a.split_counter = ctr + 5;
-    a.chunk = c->p2p_chunk;
     a.arena_cap = arena_cap;
     a.p2p_off = c->p2p_off.as<long long>();
     a.p2p_cnt = c->p2p_cnt.as<int>();
