@@ -585,18 +585,36 @@ __global__ void k_p2p_split(const uint32_t* __restrict__ counts, const int* __re
   const int chunk = p2p_chunk_of(*list_total, most, want);
   if (blockIdx.x == 0 && threadIdx.x == 0) *chunk_now = (unsigned long long)chunk;
   const int nleaves = (int)counts[1];
-  for (int leaf = blockIdx.x * blockDim.x + threadIdx.x; leaf < nleaves; leaf += gridDim.x * blockDim.x) {
-    const int cnt = p2p_cnt[leaf];
-    if (cnt <= chunk) {
-      split[leaf] = -1;
-      continue;
+  const int lane = threadIdx.x & 31;
+  // warp-aligned strides: a warp's split leaves take their places with one
+  // atomic per counter (one per leaf took 80 us where 10^5 lists are split)
+  for (int leaf0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); leaf0 < nleaves; leaf0 += gridDim.x * blockDim.x) {
+    const int leaf = leaf0 + lane;
+    const int cnt = leaf < nleaves ? p2p_cnt[leaf] : 0;
+    const int nch = cnt > chunk ? (cnt + chunk - 1) / chunk : 0;
+    const unsigned who = __ballot_sync(SFMM_FULL, nch > 0);
+    if (leaf < nleaves && nch == 0) split[leaf] = -1;
+    if (!who) continue;
+    int incl = nch;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(SFMM_FULL, incl, o);
+      if (lane >= o) incl += y;
     }
-    const int nch = (cnt + chunk - 1) / chunk;
-    const int x = (int)atomicAdd(ctr, (unsigned long long)(nch - 1));
-    const int base = (int)atomicAdd(ctr + 1, (unsigned long long)nch);
-    const int q = (int)atomicAdd(ctr + 2, 1ull);
+    const int tot = __shfl_sync(SFMM_FULL, incl, 31), nsp = __popc(who);
+    int x = 0, base = 0, q = 0;
+    if (lane == 0) {
+      x = (int)atomicAdd(ctr, (unsigned long long)(tot - nsp));
+      base = (int)atomicAdd(ctr + 1, (unsigned long long)tot);
+      q = (int)atomicAdd(ctr + 2, (unsigned long long)nsp);
+    }
+    const int before = __popc(who & lanemask_lt());
+    x = __shfl_sync(SFMM_FULL, x, 0) + incl - nch - before;
+    base = __shfl_sync(SFMM_FULL, base, 0) + incl - nch;
+    q = __shfl_sync(SFMM_FULL, q, 0) + before;
+    if (nch == 0) continue;
     if (x + nch - 1 > max_extra || base + nch > max_slots || q >= max_split) {
-      // the walk counted these exactly: more means an internal inconsistency
+      // the buffers are sized for every list: more means an internal inconsistency
       split[leaf] = -1;
       set_status(status, SFMM_ST_INTERNAL);
       continue;
@@ -667,13 +685,14 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   // long lists: slots, extra items and split leaves are counted by the split
   // pass on the device; the buffers are sized from bounds on the host (a list
   // of cnt > chunk entries takes ceil(cnt / chunk) <= 2 cnt / chunk slots, and
-  // entries / chunk is at most arena / option or 9/8 want), with no wait for
+  // entries / chunk is at most arena / maximum or 9/8 want), with no wait for
   // the walk
+  const int most = c->p2p_chunk;
   const int64_t arena_cap = (int64_t)(c->arena.bytes / sizeof(int));
   const int nslots =
-      (int)std::min<int64_t>(std::max<int64_t>(2 * arena_cap / c->p2p_chunk, 3 * (int64_t)want) + 2, INT32_MAX / 2);
+      (int)std::min<int64_t>(std::max<int64_t>(2 * arena_cap / most, 3 * (int64_t)want) + 2, INT32_MAX / 2);
   const int nsplit = (int)std::min<int64_t>(
-      std::min<int64_t>(c->graph_mode ? c->n : nl, std::max<int64_t>(arena_cap / (c->p2p_chunk + 1), 2 * (int64_t)want) + 1),
+      std::min<int64_t>(c->graph_mode ? c->n : nl, std::max<int64_t>(arena_cap / (most + 1), 2 * (int64_t)want) + 1),
       nslots);
   const int nextra = nslots;
   int lmax = c->leaf_size;
@@ -686,7 +705,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   const int sblocks = std::max(1, std::min((nl_b + 255) / 256, 8 * num_sms(c->device)));
   k_p2p_split<<<sblocks, 256, 0, c->stream>>>(c->d_counts, c->p2p_cnt.as<int>(), c->p2p_split.as<int>(),
                                                      c->p2p_extra.as<int2>(), c->p2p_slist.as<int>(), ctr + 11,
-                                                     nextra, nslots, nsplit, c->p2p_chunk, want, ctr + 9, ctr + 7, c->d_status);
+                                                     nextra, nslots, nsplit, most, want, ctr + 9, ctr + 7, c->d_status);
   ++c->nlaunch;
   SFMM_CUDA_TRY(cudaGetLastError());
   P2PArgs a{};
@@ -757,7 +776,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   SFMM_CUDA_TRY(cudaGetLastError());
   {
     // split leaves (their count is on the device): a persistent grid
-    const int cblocks = std::min(2 * num_sms(c->device), (nsplit + 7) / 8 + 1);
+    const int cblocks = std::min(6 * num_sms(c->device), (nsplit + 7) / 8 + 1);
     if (f32) k_p2p_combine<true><<<cblocks, 256, 0, c->stream>>>(a);
     else k_p2p_combine<false><<<cblocks, 256, 0, c->stream>>>(a);
     ++c->nlaunch;

@@ -24,7 +24,10 @@
 // Default of the option "p2p_chunk": neighbour lists longer than this many
 // entries are split into chunks of it, each a separate near-field work item
 // (long lists would otherwise leave one warp working alone at the end of the
-// pass).
+// pass).  Longer items are slower even where the lists are long enough for
+// eight per resident warp: at most 2048 instead of 256, the near field of the
+// 256-system ensemble went from 13.1 to 13.7 ms, of the 2e6 binary from 3.89
+// to 4.00 ms.
 #define SFMM_P2P_CHUNK_DEFAULT 256
 
 namespace sfmm {
