@@ -175,8 +175,13 @@ __device__ __forceinline__ void reduce_sums(const T (&C)[N], T* s, int lane) {
 
 // Acceptance test of Sect. 3: accept iff (l_t + l_s) < theta d and not
 // d < l_t + l_s + R_kern max(h_t, h_s).
+// on: whether the lane holds a pair to test (else false).  Branch-free but for
+// the float64 path: the walk is half decisions, and with early returns it took
+// 14.65 ms instead of 13.79 on the 1.6e7 cloud, 0.89 instead of 0.79 at 1e5
+// particles and order 4.
 __device__ __forceinline__ bool decide(const float4& hiA, const float4& loA, const float4& hiB, const float4& loB,
-                                       int A, int B, const WalkArgs& a, int& nfb, float& dx, float& dy, float& dz) {
+                                       int A, int B, const WalkArgs& a, int& nfb, float& dx, float& dy, float& dz,
+                                       bool on) {
   dx = df_diff(hiB.x, loB.x, hiA.x, loA.x);
   dy = df_diff(hiB.y, loB.y, hiA.y, loA.y);
   dz = df_diff(hiB.z, loB.z, hiA.z, loA.z);
@@ -190,20 +195,22 @@ __device__ __forceinline__ bool decide(const float4& hiA, const float4& loA, con
   const float rhs = fmaf(2.0f, hm, ls);
   const float rhs2 = rhs * rhs;
   const float m2 = d2 - rhs2, t2 = 1e-5f * (d2 + rhs2);
-  if (d2 >= 1e-30f && d2 <= 1e30f) {
-    if (m1 < -t1 || m2 < -t2) return false;
-    if (m1 > t1 && m2 > t2) return true;
+  const bool ok = (d2 >= 1e-30f) & (d2 <= 1e30f);
+  const bool no = (m1 < -t1) | (m2 < -t2);
+  bool acc = (m1 > t1) & (m2 > t2);
+  if (on & (!ok | !(no | acc))) {
+    ++nfb;
+    const double ddx = dsub(a.ncx[B], a.ncx[A]);
+    const double ddy = dsub(a.ncy[B], a.ncy[A]);
+    const double ddz = dsub(a.ncz[B], a.ncz[A]);
+    const double dd = __dsqrt_rn(dadd(dadd(dmul(ddx, ddx), dmul(ddy, ddy)), dmul(ddz, ddz)));
+    const double lsd = dadd(a.nsize[A], a.nsize[B]);
+    const double hmd = fmax(a.nhmax[A], a.nhmax[B]);
+    const bool mac = lsd < dmul(a.theta, dd);
+    const bool soft = dd < dadd(lsd, dmul(SFMM_RKERN, hmd));
+    acc = mac && !soft;
   }
-  ++nfb;
-  const double ddx = dsub(a.ncx[B], a.ncx[A]);
-  const double ddy = dsub(a.ncy[B], a.ncy[A]);
-  const double ddz = dsub(a.ncz[B], a.ncz[A]);
-  const double dd = __dsqrt_rn(dadd(dadd(dmul(ddx, ddx), dmul(ddy, ddy)), dmul(ddz, ddz)));
-  const double lsd = dadd(a.nsize[A], a.nsize[B]);
-  const double hmd = fmax(a.nhmax[A], a.nhmax[B]);
-  const bool mac = lsd < dmul(a.theta, dd);
-  const bool soft = dd < dadd(lsd, dmul(SFMM_RKERN, hmd));
-  return mac && !soft;
+  return on & acc;
 }
 
 // One node-node interaction (target centre A, source node s) accumulated
@@ -413,7 +420,7 @@ __device__ __forceinline__ void m2l_eval(int s, const float4& hiA, const float4&
 __device__ __forceinline__ bool decide(const float4& hiA, const float4& loA, const float4& hiB, const float4& loB,
                                        int A, int B, const WalkArgs& a, int& nfb) {
   float dx, dy, dz;
-  return decide(hiA, loA, hiB, loB, A, B, a, nfb, dx, dy, dz);
+  return decide(hiA, loA, hiB, loB, A, B, a, nfb, dx, dy, dz, true);
 }
 
 }  // namespace sfmm

@@ -419,15 +419,9 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
             rB = a.nright[s];
           }
         }
-        bool acc = false, open = false;
-        float rx = 0.f, ry = 0.f, rz = 0.f;
-        if (s >= 0) {
-          if (s == A) open = true;
-          else {
-            acc = decide(hiA, loA, hiB, loB, A, s, a, st_fb, rx, ry, rz);
-            open = !acc;
-          }
-        }
+        float rx, ry, rz;
+        bool acc = decide(hiA, loA, hiB, loB, A, s, a, st_fb, rx, ry, rz, (s >= 0) & (s != A));
+        const bool open = (s >= 0) & !acc;
         if constexpr (SYM) {
           // the node processed first evaluates the pair for both sides
           // (leaves run last; ties within a launch go to the smaller id)
@@ -452,11 +446,8 @@ __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1
           const int add = __popc(b1) + __popc(b2);
           if (open) {
             const int pos = nn + __popc(b1 & lt) + __popc(b2 & lt);
-            if (sleaf) cfw[pos] = s;
-            else {
-              cfw[pos] = s + 1;
-              cfw[pos + 1] = rB;
-            }
+            cfw[pos] = sleaf ? s : s + 1;
+            if (sint) cfw[pos + 1] = rB;
           }
           nn += add;
         } else {
@@ -734,9 +725,9 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
   // (each record load serves both children's decisions, at fewer warps per
   // SM); 0 chooses 2 while the walk's records (geometry, moments,
   // coefficients, list offsets) take at most twice the L2, else 3
-  // (measured on GB300: 2 is faster on the 10^6 Plummer sphere, 1.21 against
-  // 1.32 ms, records 64 MB, and on the 2x10^6 binary, 2.11 against 2.17 ms,
-  // records 127 MB; 3 on the 1.6x10^7 cloud, 16.3 against 17.4 ms, 1 GB)
+  // (measured on GB300: 2 is faster on the 10^6 Plummer sphere, 1.14 against
+  // 1.28 ms, records 64 MB, and on the 2x10^6 binary, 1.96 against 1.97 ms,
+  // records 127 MB; 3 on the 1.6x10^7 cloud, 14.7 against 15.9 ms, 1 GB)
   int sched = SYM ? 1 : c->schedule;
   if (sched == 0) {
     int l2 = 0;
