@@ -592,6 +592,11 @@ static __device__ const unsigned short sfmm_l2l_steps_0[1][32] = {
   {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
 static const int sfmm_moment_mi_0[1][3] = {{0,0,0}};
 
+#define SFMM_MT_0 1  /* steps of the M2M translation */
+static __device__ const unsigned short sfmm_m2m_steps_0[1][32] = {
+  {0, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
+static __device__ const unsigned short sfmm_moment_exp_0[1] = {0};
+
 template <typename T> __device__ __forceinline__ void sfmm_fold_0(const T* Q, T* q) {
   q[0] = Q[0];
 }
@@ -727,6 +732,12 @@ static __device__ const unsigned short sfmm_l2l_steps_1[3][32] = {
   {514, 65535, 65535, 65535, 520, 522, 523, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
   {771, 65535, 65535, 65535, 777, 779, 780, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
 static const int sfmm_moment_mi_1[4][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}};
+
+#define SFMM_MT_1 2  /* steps of the M2M translation */
+static __device__ const unsigned short sfmm_m2m_steps_1[2][32] = {
+  {0, 1, 2, 3, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 256, 512, 768, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
+static __device__ const unsigned short sfmm_moment_exp_1[4] = {0, 1, 8, 64};
 
 template <typename T> __device__ __forceinline__ void sfmm_fold_1(const T* Q, T* q) {
   q[0] = Q[0];
@@ -1079,6 +1090,14 @@ static __device__ const unsigned short sfmm_l2l_steps_2[9][32] = {
   {2056, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 2071, 2074, 2075, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
   {2313, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 2328, 2331, 2332, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
 static const int sfmm_moment_mi_2[10][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}, {2,0,0}, {1,1,0}, {1,0,1}, {0,2,0}, {0,1,1}, {0,0,2}};
+
+#define SFMM_MT_2 4  /* steps of the M2M translation */
+static __device__ const unsigned short sfmm_m2m_steps_2[4][32] = {
+  {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 256, 512, 768, 257, 258, 259, 514, 515, 771, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 1024, 513, 769, 1792, 770, 2304, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 1280, 1536, 65535, 2048, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
+static __device__ const unsigned short sfmm_moment_exp_2[10] = {0, 1, 8, 64, 2, 9, 65, 16, 72, 128};
 
 template <typename T> __device__ __forceinline__ void sfmm_fold_2(const T* Q, T* q) {
   q[0] = Q[0];
@@ -1941,6 +1960,18 @@ static __device__ const unsigned short sfmm_l2l_steps_3[19][64] = {
   {4626, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 4655, 4659, 4660, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
   {4883, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 4912, 4916, 4917, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
 static const int sfmm_moment_mi_3[20][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}, {2,0,0}, {1,1,0}, {1,0,1}, {0,2,0}, {0,1,1}, {0,0,2}, {3,0,0}, {2,1,0}, {2,0,1}, {1,2,0}, {1,1,1}, {1,0,2}, {0,3,0}, {0,2,1}, {0,1,2}, {0,0,3}};
+
+#define SFMM_MT_3 8  /* steps of the M2M translation */
+static __device__ const unsigned short sfmm_m2m_steps_3[8][32] = {
+  {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 256, 512, 768, 257, 258, 259, 514, 515, 771, 260, 261, 262, 263, 264, 265, 519, 520, 521, 777, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 1024, 513, 769, 1792, 770, 2304, 1025, 516, 772, 517, 518, 774, 1794, 775, 776, 2307, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 1280, 1536, 65535, 2048, 65535, 2560, 1026, 1027, 1282, 773, 1539, 4096, 1795, 2051, 4864, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 1281, 1537, 1793, 1283, 2305, 65535, 2050, 2306, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 2816, 3072, 3328, 1538, 3840, 65535, 4352, 4608, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 2049, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 3584, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
+static __device__ const unsigned short sfmm_moment_exp_3[20] = {0, 1, 8, 64, 2, 9, 65, 16, 72, 128, 3, 10, 66, 17, 73, 129, 24, 80, 136, 192};
 
 template <typename T> __device__ __forceinline__ void sfmm_fold_3(const T* Q, T* q) {
   q[0] = Q[0];
@@ -3839,6 +3870,22 @@ static __device__ const unsigned short sfmm_l2l_steps_4[34][96] = {
   {8481, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 8530, 8535, 8536, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
   {8738, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 8787, 8792, 8793, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
 static const int sfmm_moment_mi_4[35][3] = {{0,0,0}, {1,0,0}, {0,1,0}, {0,0,1}, {2,0,0}, {1,1,0}, {1,0,1}, {0,2,0}, {0,1,1}, {0,0,2}, {3,0,0}, {2,1,0}, {2,0,1}, {1,2,0}, {1,1,1}, {1,0,2}, {0,3,0}, {0,2,1}, {0,1,2}, {0,0,3}, {4,0,0}, {3,1,0}, {3,0,1}, {2,2,0}, {2,1,1}, {2,0,2}, {1,3,0}, {1,2,1}, {1,1,2}, {1,0,3}, {0,4,0}, {0,3,1}, {0,2,2}, {0,1,3}, {0,0,4}};
+
+#define SFMM_MT_4 12  /* steps of the M2M translation */
+static __device__ const unsigned short sfmm_m2m_steps_4[12][64] = {
+  {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21, 22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 256, 512, 768, 257, 258, 259, 514, 515, 771, 260, 261, 262, 263, 264, 265, 519, 520, 521, 777, 266, 267, 268, 269, 270, 271, 272, 273, 274, 275, 528, 529, 530, 531, 787, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 1024, 513, 769, 1792, 770, 2304, 1025, 516, 772, 517, 518, 774, 1794, 775, 776, 2307, 1028, 522, 778, 523, 524, 780, 525, 526, 527, 783, 1799, 784, 785, 786, 2313, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 1280, 1536, 65535, 2048, 65535, 2560, 1026, 1027, 1282, 773, 1539, 4096, 1795, 2051, 4864, 2561, 1029, 1030, 1031, 779, 1033, 1287, 781, 782, 1545, 4098, 1800, 1801, 2057, 4867, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 1281, 1537, 1793, 1283, 2305, 65535, 2050, 2306, 65535, 5120, 1284, 1540, 1285, 1032, 1542, 1797, 1288, 1289, 2310, 7680, 2055, 2056, 2312, 8704, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 2816, 3072, 3328, 1538, 3840, 65535, 4352, 4608, 65535, 65535, 2562, 2563, 1796, 1286, 2308, 3330, 1543, 1544, 3843, 65535, 4099, 2311, 4611, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 2049, 65535, 65535, 65535, 65535, 65535, 65535, 2817, 3073, 2818, 1541, 3075, 4097, 1798, 2054, 4865, 65535, 4354, 4355, 4866, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 3584, 65535, 65535, 65535, 65535, 65535, 65535, 5376, 5632, 3329, 2052, 3841, 6656, 2053, 2309, 7424, 65535, 7936, 4610, 8448, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 5888, 2819, 6400, 65535, 3331, 3587, 65535, 65535, 65535, 8192, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 3074, 65535, 65535, 3586, 3842, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 3585, 65535, 65535, 4353, 4609, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535},
+  {65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 6144, 65535, 65535, 6912, 7168, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535, 65535}};
+static __device__ const unsigned short sfmm_moment_exp_4[35] = {0, 1, 8, 64, 2, 9, 65, 16, 72, 128, 3, 10, 66, 17, 73, 129, 24, 80, 136, 192, 4, 11, 67, 18, 74, 130, 25, 81, 137, 193, 32, 88, 144, 200, 256};
 
 template <typename T> __device__ __forceinline__ void sfmm_fold_4(const T* Q, T* q) {
   q[0] = Q[0];

@@ -204,6 +204,22 @@ def gen_m2m(p):
     return "\n".join(lines)
 
 
+def gen_m2m_steps(p):
+    """Lane-parallel M2M: step k of moment j holds the k-th term of gen_m2m's
+    sum, monomial + 256 child moment (0xffff: no more terms); exponents of
+    moment j as a + 8 b + 64 c."""
+    IQ = idx_of(p)
+    rows = [[IQ[sub(a, b)] + 256 * IQ[b] for b in mis(p) if geq(a, b)] for a in mis(p)]
+    n, steps = len(rows), max(len(r) for r in rows)
+    stride = (n + 31) // 32 * 32
+    body = ",\n  ".join("{" + ", ".join("%d" % (rows[j][k] if j < n and k < len(rows[j]) else 0xffff)
+                                         for j in range(stride)) + "}" for k in range(steps))
+    exps = ", ".join("%d" % (g[0] + 8 * g[1] + 64 * g[2]) for g in mis(p))
+    return ("#define SFMM_MT_%d %d  /* steps of the M2M translation */\n" % (p, steps)
+            + "static __device__ const unsigned short sfmm_m2m_steps_%d[%d][%d] = {\n  %s};\n" % (p, steps, stride, body)
+            + "static __device__ const unsigned short sfmm_moment_exp_%d[%d] = {%s};\n" % (p, n, exps))
+
+
 def gen_tables(p):
     """Lane-parallel L2L: target coefficient j is its own source plus
     h^(gamma_i - beta_j)/()! C_i over the other sources i of its block (M or F)
@@ -391,6 +407,7 @@ def main():
         out.append(gen_m2m(p))
         out.append("")
         out.append(gen_tables(p))
+        out.append(gen_m2m_steps(p))
         out.append(gen_fold(p))
         out.append("")
         out.append(gen_m2l_fold(p))

@@ -980,6 +980,7 @@ __global__ void k_leaf_geom(const uint32_t* __restrict__ counts, const int* __re
   #pragma unroll
     for (int c = 0; c < 6; ++c) ek[c] = dkey(ev[c]);
     int ei[6] = {f, f, f, f, f, f};
+#pragma unroll 4
     for (int i = f; i < f + cnt; ++i) {
       const double m = pm[i];
       M = dadd(M, m);
@@ -1018,6 +1019,7 @@ __global__ void k_leaf_geom(const uint32_t* __restrict__ counts, const int* __re
     QT acc[NQ];
   #pragma unroll
     for (int k = 0; k < NQ; ++k) acc[k] = QT(0);
+#pragma unroll 2
     for (int i = f; i < f + cnt; ++i) {
       const double dx = dsub(px[i], cx), dy = dsub(py[i], cy), dz = dsub(pz[i], cz);
       const float fx = __double2float_rn(dx), fy = __double2float_rn(dy), fz = __double2float_rn(dz);
@@ -1041,10 +1043,11 @@ __global__ void k_leaf_geom(const uint32_t* __restrict__ counts, const int* __re
 // count and the axis-extreme particles (the left child's on ties).  The
 // children's records are read through L2: another thread of this launch may
 // have written them.
+// shift: where the children's centres lie from v's (left 3, right 3), or null.
 template <int P, typename QT>
 __device__ __forceinline__ void upward_node(int v, int R, double* ncx, double* ncy, double* ncz, double* nmass,
                                             double* nhmax, int* nlu, double* extv, int* exti, double* Qd,
-                                            float* Qf) {
+                                            float* Qf, double* shift = nullptr) {
   const int L = v + 1;
   // every load first: the stores below may alias them as far as the
   // compiler knows, and loads left after a store would wait for the work
@@ -1079,6 +1082,14 @@ __device__ __forceinline__ void upward_node(int v, int R, double* ncx, double* n
   ncx[v] = cx;
   ncy[v] = cy;
   ncz[v] = cz;
+  if (shift) {
+    shift[0] = cLx - cx;
+    shift[1] = cLy - cy;
+    shift[2] = cLz - cz;
+    shift[3] = cRx - cx;
+    shift[4] = cRy - cy;
+    shift[5] = cRz - cz;
+  }
   if constexpr (P >= 0) {
     QT qp[NQ];
   #pragma unroll
@@ -1109,6 +1120,109 @@ __device__ __forceinline__ void upward_node(int v, int R, double* ncx, double* n
 // GB300: computing the top of the tree -- the ~1500 nodes of more than 10^3
 // particles, 23 levels deep -- level by level in one block after a climb
 // that stops below it was slower, 0.18 against 0.13 ms.)
+// The climb with FP64 moments, warp by warp.  An FP64 instruction takes the
+// pipe about 80 cycles whatever the active lanes, and near the top of the tree
+// one or two lanes of a warp climb: up to four of them have their moments
+// translated one node after the other by the whole warp, a moment per lane (12
+// steps of FP64 work for p = 2, 28 for p = 3, instead of 88 and 230 for a
+// thread translating all its moments); more climb side by side as in k_upward.
+// Same operations in the same order, so the same moments bit for bit.
+template <int P>
+__global__ void __launch_bounds__(128) k_upward_fp64(const uint32_t* __restrict__ counts,
+                                                     const int* __restrict__ leaf_node,
+                                                     const int* __restrict__ nparent, const int* __restrict__ nright,
+                                                     double* ncx, double* ncy, double* ncz, double* nmass,
+                                                     double* nhmax, int* nlu, int* flags, double* extv, int* exti,
+                                                     double* Qd, float* Qf) {
+  using M = MomOps<P>;
+  constexpr int NQ = M::NQ, NQS = (NQ + 3) & ~3, NB = (NQ + 31) / 32;
+  __shared__ double s_g[4][2][NQ], s_q[4][2][NQ];  // per warp: both children's shift monomials and moments
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nleaves = (int)counts[1];
+  for (int q0 = blockIdx.x * blockDim.x + 32 * warp; q0 < nleaves; q0 += gridDim.x * blockDim.x) {
+    int v = q0 + lane < nleaves ? nparent[leaf_node[q0 + lane]] : -1;
+    while (__any_sync(SFMM_FULL, v >= 0)) {
+      bool go = false;
+      int R = 0, up = -1;
+      double sh[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      if (v >= 0) {
+        R = nright[v];
+        up = nparent[v];
+        cuda::atomic_ref<int, cuda::thread_scope_device> arrive(flags[v]);
+        go = arrive.fetch_add(1, cuda::memory_order_acq_rel) != 0;
+      }
+      if (go) upward_node<-1, double>(v, R, ncx, ncy, ncz, nmass, nhmax, nlu, extv, exti, Qd, Qf, sh);
+      unsigned act = __ballot_sync(SFMM_FULL, go);
+      if (__popc(act) > 4) {
+        if (go) {
+          double qc[NQ], g[NQ], qp[NQ];
+#pragma unroll
+          for (int k = 0; k < NQ; ++k) qp[k] = 0.0;
+          load_moments<NQ>(v + 1, qc, Qd, Qf);
+          M::mono(sh[0], sh[1], sh[2], g);
+          M::m2m(g, qc, qp);
+          load_moments<NQ>(R, qc, Qd, Qf);
+          M::mono(sh[3], sh[4], sh[5], g);
+          M::m2m(g, qc, qp);
+          store_moments<NQ>(v, qp, 0.0, Qd, Qf);
+        }
+      } else {
+        __syncwarp();  // what the climbing lanes acquired is the warp's to read
+        while (act) {
+          const int o = __ffs(act) - 1;
+          act &= act - 1;
+          const int w = __shfl_sync(SFMM_FULL, v, o), wr = __shfl_sync(SFMM_FULL, R, o);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const double x = __shfl_sync(SFMM_FULL, sh[3 * c], o), y = __shfl_sync(SFMM_FULL, sh[3 * c + 1], o),
+                         z = __shfl_sync(SFMM_FULL, sh[3 * c + 2], o);
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+              const int k = lane + 32 * b;
+              if (k < NQ) {
+                s_q[warp][c][k] = __ldcg(&Qd[(int64_t)(c ? wr : w + 1) * NQ + k]);
+                // the monomial by gen_mono's recurrence: z factors, then y, then x
+                const int e = M::exponents()[k], ez = e >> 6, ey = (e >> 3) & 7, ex = e & 7;
+                double m = 1.0;
+#pragma unroll
+                for (int s = 0; s < P; ++s) {
+                  if (s < ex + ey + ez) {
+                    const bool inz = s < ez, iny = s < ez + ey;
+                    const double u = inz ? z : iny ? y : x;
+                    const int f = s + 1 - (inz ? 0 : iny ? ez : ez + ey);
+                    m *= f == 1 ? u : u * (f == 2 ? 1.0 / 2.0 : f == 3 ? 1.0 / 3.0 : 1.0 / 4.0);
+                  }
+                }
+                s_g[warp][c][k] = m;
+              }
+            }
+          }
+          __syncwarp();
+#pragma unroll
+          for (int b = 0; b < NB; ++b) {
+            const int k = lane + 32 * b;
+            if (k < NQ) {
+              double s = 0.0;
+#pragma unroll
+              for (int c = 0; c < 2; ++c)
+                for (int t = 0; t < M::MT; ++t) {
+                  const int e = M::steps()[t * M::MS + k];
+                  if (e != 0xffff) s = fma(s_g[warp][c][e & 255], s_q[warp][c][e >> 8], s);
+                }
+              Qd[(int64_t)w * NQ + k] = s;
+              Qf[(int64_t)w * NQS + k] = (float)s;
+            }
+          }
+          if (lane < NQS - NQ) Qf[(int64_t)w * NQS + NQ + lane] = 0.0f;
+          __syncwarp();
+        }
+      }
+      __syncwarp();
+      v = go ? up : -1;
+    }
+  }
+}
+
 template <int P, typename QT>
 __global__ void k_upward(const uint32_t* __restrict__ counts, const int* __restrict__ leaf_node, const int* __restrict__ nparent,
                          const int* __restrict__ nright, double* ncx, double* ncy, double* ncz, double* nmass,
@@ -1227,6 +1341,7 @@ __global__ void k_size_leaf(const uint32_t* __restrict__ counts, const int* __re
     // offsets too small or too large for that bound take every particle
     float best = -1.0f;
     int bi = f;
+#pragma unroll 8
     for (int i = f; i < f + cnt; ++i) {
       const float4 r = prel[i];
       const float d2 = fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z));
@@ -1237,6 +1352,7 @@ __global__ void k_size_leaf(const uint32_t* __restrict__ counts, const int* __re
     }
     double l2 = exact_d2(px[bi], py[bi], pz[bi], cx, cy, cz);
     const float thr = (best > 1e-30f && best < 1e30f) ? best * (1.0f - 4e-6f) : -1.0f;
+#pragma unroll 8
     for (int i = f; i < f + cnt; ++i) {
       const float4 r = prel[i];
       if (i != bi && fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z)) >= thr)
@@ -1505,7 +1621,13 @@ static int geom_upward_t(sfmm_ctx* c, int nqs) {
   ++c->nlaunch;
   // the second child to finish climbs on (arrival flags cleared by the leaf
   // numbering pass)
-  k_upward<P, QT><<<leaf_grid(c), 128, 0, st>>>(c->d_counts, c->leaf_node.as<int>(), c->nparent.as<int>(), c->nright.as<int>(),
+  if constexpr (P >= 1 && std::is_same<QT, double>::value)
+    k_upward_fp64<P><<<leaf_grid(c), 128, 0, st>>>(
+        c->d_counts, c->leaf_node.as<int>(), c->nparent.as<int>(), c->nright.as<int>(), c->ncx.as<double>(),
+        c->ncy.as<double>(), c->ncz.as<double>(), c->nmass.as<double>(), c->nhmax.as<double>(), c->nlu.as<int>(),
+        c->flags.as<int>(), c->n_extv.as<double>(), c->n_exti.as<int>(), c->Qd.as<double>(), c->Qf.as<float>());
+  else
+    k_upward<P, QT><<<leaf_grid(c), 128, 0, st>>>(c->d_counts, c->leaf_node.as<int>(), c->nparent.as<int>(), c->nright.as<int>(),
                                                  c->ncx.as<double>(), c->ncy.as<double>(), c->ncz.as<double>(),
                                                  c->nmass.as<double>(), c->nhmax.as<double>(), c->nlu.as<int>(),
                                                  c->flags.as<int>(), c->n_extv.as<double>(), c->n_exti.as<int>(),

@@ -1,7 +1,7 @@
 """Paths that small sets and batches take: the one-block sort and scan at the
 edges of their ranges (4096 particles, 8192 values), sums over slices of 8192
-particles of a system, and neighbour lists cut finer than the option when the
-lists are few."""
+particles of a system, neighbour lists cut finer than the option when the lists
+are few, and FP64 moments translated a moment per lane where few lanes climb."""
 import math
 
 import numpy as np
@@ -62,3 +62,29 @@ def test_few_lists_are_cut_finer(prec, n, leaf):
         acc, pot = (t.cpu().numpy() for t in s.gravity(0.4, 2))
         s.close()
         assert acc_rel(acc, a_o).max() <= tol and pot_rel(pot, p_o).max() <= tol
+
+
+@pytest.mark.parametrize("order", [1, 2, 3, 4])
+@pytest.mark.parametrize("n,leaf", [(2, 1), (5, 1), (40, 1), (300, 2), (3000, 1), (20000, 16)])
+def test_moments_of_the_climb(order, n, leaf):
+    """The build's FP64 moments (warp-wide translation for up to four climbing
+    lanes, a thread per node beyond) against the pass that translates every
+    node by a thread: the same operations, so 1e-14 of the moments' scale
+    leaves room for the leaf sums only."""
+    pos, m, h = workloads.plummer(n, 60 + n)
+    ref = solver("fp64")
+    ref.build(pos, m, h, leaf)
+    ref.gravity(0.8, 0)
+    ref.build(pos, m, h, leaf)  # moments of order 0: the export makes its own
+    Qr, mi = ref.moments(order)
+    t = ref.tree()
+    s = solver("fp64")
+    s.build(pos, m, h, leaf)
+    s.gravity(0.8, order)
+    s.build(pos, m, h, leaf)  # moments of this order on the way up
+    Q, _ = s.moments(order)
+    ref.close()
+    s.close()
+    for k, deg in enumerate(np.asarray(mi).sum(1)):
+        scale = t["mass"] * (t["size"] + 1e-16) ** deg + (1e-15 * t["mass"] if deg == 1 else 0.0)
+        assert (np.abs(Q[:, k] - Qr[:, k]) <= 1e-14 * scale + 1e-30).all(), (order, k)
