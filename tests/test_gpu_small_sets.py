@@ -28,6 +28,23 @@ def test_sorted_order_and_tree(n):
         assert np.array_equal(t[k], getattr(o, k)), k
 
 
+@pytest.mark.parametrize("sizes", [[6143], [6144], [6145], [22529], [150001], [2047, 1, 4097, 6144, 300]])
+def test_sort_tiles(sizes):
+    # tiles of 2048 keys, one per block, and the passes over the system index
+    parts = [workloads.plummer(n, 70 + n) for n in sizes]
+    for p in parts:
+        n = len(p[1])
+        p[0][n // 3:n // 2] = p[0][n // 3]
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    pos, m, h = (np.concatenate([p[q] for p in parts]) for q in range(3))
+    s = solver("fp32")
+    s.build_batch(off, pos, m, h, np.full(len(sizes), 8, np.int32))
+    perm = s.tree()["perm"]
+    s.close()
+    want = [a + oracle.Tree(*p, 8, p=0).perm for a, p in zip(off, parts)]
+    assert np.array_equal(perm, np.concatenate(want))
+
+
 def test_sums_of_sliced_systems():
     sizes = [1, 8191, 8192, 8193, 20001]
     parts = [workloads.plummer(k, 50 + k) for k in sizes]
