@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
               // the owner: the first lane whose inclusive count exceeds k
               int o = 0;
 #pragma unroll
-              for (int w = 16; w > 0; w >>= 1)
-                if (__shfl_sync(SFMM_FULL, incl, o + w - 1) <= k) o += w;
+              for (int b = 16; b > 0; b >>= 1)
+                if (__shfl_sync(SFMM_FULL, incl, o + b - 1) <= k) o += b;
               const unsigned om0 = __shfl_sync(SFMM_FULL, m0, o), om1 = __shfl_sync(SFMM_FULL, m1, o);
               const int rank = k - __shfl_sync(SFMM_FULL, own0, o);
               const int osteps = __shfl_sync(SFMM_FULL, steps, o), oph = __shfl_sync(SFMM_FULL, ph, o),
