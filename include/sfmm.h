@@ -118,9 +118,10 @@ int sfmm_set_stream(sfmm_ctx* ctx, void* stream);
  *                    2 one launch in which a warp takes the next node whose
  *                    parent is done from a queue; 3 the same with both
  *                    children of a node taken by one warp (their common
- *                    inherited list read once); 0 (default) chooses 2 when
- *                    the walk's per-node records take at most twice the L2
- *                    cache, else 3; bitwise the same results
+ *                    inherited list read once); 0 (default) chooses by
+ *                    form, order and how the walk's per-node records compare
+ *                    with the L2 cache (2 for sets that fit, 3 for larger ones
+ *                    at the orders it suits); bitwise the same results
  *   "tree"           0 (default): binary radix tree over Morton keys (Sect. 3);
  *                    1: centre-of-mass-pivot kd tree (Sect. 3; single
  *                    systems only, sfmm_build_batch returns ENOTIMPL)

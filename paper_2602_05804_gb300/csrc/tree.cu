@@ -386,7 +386,7 @@ __global__ void k_morton(const double* __restrict__ pos, int n, const double* __
 // (key, input index) in shared memory -- the pairs are distinct, so the order
 // is the stable one.  The radix passes are bound by latency there (70 us in all
 // at 1000 particles, where this takes about 10); the network grows faster
-// (about 40 us at 4096, 200 us at 16,384 against 85).
+// (about 40 us at 4096, 200 us at 16,384; the passes take 66 us at 10^4).
 #define SMALL_SORT_NT 1024
 #define SMALL_SORT_MAX 4096
 
@@ -1159,7 +1159,9 @@ __device__ __forceinline__ void upward_node(int v, int R, double* ncx, double* n
 // translated one node after the other by the whole warp, a moment per lane (12
 // steps of FP64 work for p = 2, 28 for p = 3, instead of 88 and 230 for a
 // thread translating all its moments); more climb side by side as in k_upward.
-// Same operations in the same order, so the same moments bit for bit.
+// Same operations in the same order, so the same moments bit for bit.  Build,
+// before and now: 0.67 and 0.50 ms (10^5 particles, p = 3), 0.95 and 0.85 (10^6,
+// p = 2), 0.39 and 0.36 (13,000).
 template <int P>
 __global__ void __launch_bounds__(128) k_upward_fp64(const uint32_t* __restrict__ counts,
                                                      const int* __restrict__ leaf_node,

@@ -724,10 +724,15 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
   // depth; 2 readiness queue of nodes; 3 readiness queue of sibling pairs
   // (each record load serves both children's decisions, at fewer warps per
   // SM); 0 chooses 2 while the walk's records (geometry, moments,
-  // coefficients, list offsets) take at most twice the L2, else 3
-  // (measured on GB300: 2 is faster on the 10^6 Plummer sphere, 1.14 against
-  // 1.28 ms, records 64 MB, and on the 2x10^6 binary, 1.96 against 1.97 ms,
-  // records 127 MB; 3 on the 1.6x10^7 cloud, 14.7 against 15.9 ms, 1 GB)
+  // coefficients, list offsets) fit the L2, else 3.  FP32 form up to second
+  // order (the pair kernel runs five blocks per SM): at 0.85 of the L2 (Plummer
+  // spheres, theta 0.5, p = 2, queue of nodes and of pairs: 61 MB 1.09 and 1.19
+  // ms, 104 MB 1.72 and 1.73, 122 MB 1.98 and 1.96, the binary's 122 MB 1.91
+  // and 1.84, 183 MB 2.86 and 2.75, 487 MB 7.6 and 6.9).  Third order: never
+  // (the pair kernel's sums leave it fewer warps: 226 MB 3.12 and 3.96 ms,
+  // 452 MB 6.19 and 7.77).  Otherwise at twice the L2 (p = 4, 165 MB 2.06 and
+  // 2.28, 331 MB 5.57 and 5.70, 661 MB 11.1 both; FP64 form, p = 2, 290 MB
+  // 24.6 and 24.5)
   int sched = SYM ? 1 : c->schedule;
   if (sched == 0) {
     int l2 = 0;
@@ -736,7 +741,8 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
     // source row, coefficients
     const size_t mom = (F32 ? 4 : 8) * (size_t)row_len<P, F32>();
     const size_t per_node = 48 + mom + 8 * (size_t)tstride;
-    sched = ((double)per_node * nn <= 2.0 * (double)l2) ? 2 : 3;
+    const double fit = (F32 && P <= 2) ? 0.85 : 2.0;
+    sched = ((F32 && P == 3) || (double)per_node * nn <= fit * (double)l2) ? 2 : 3;
   }
   // a captured step runs on the counts of each replay's own build: node- and
   // leaf-indexed buffers are sized for the bounds (2n nodes, n leaves), and
