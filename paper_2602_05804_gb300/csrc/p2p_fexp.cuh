@@ -80,12 +80,14 @@ __device__ __forceinline__ void m4_add(double r, double ri, double ri3, double2 
                g3 = in1 ? 0.5 : -1.0 / 6.0;
   const double p0 = in1 ? -1.4 : -1.6, p2 = in1 ? 2.0 / 3.0 : 4.0 / 3.0, p3 = in1 ? 0.0 : -1.0,
                p4 = in1 ? -0.3 : 0.3, p5 = in1 ? 0.1 : -1.0 / 30.0;
-  // outside 2h the polynomials take no part: 1/r^3 and -1/r
+  // outside 2h the polynomials take no part: 1/r^3 and -1/r; inside h 1/r^3
+  // takes none (selected, not multiplied by zero: it overflows where r < 2e-103)
   const double hv = out ? 0.0 : hinv.x, hv3 = out ? 0.0 : hinv.y, qq = out ? 0.0 : q;
-  const double cg = in1 ? 0.0 : (out ? 1.0 : -1.0 / 15.0), cp = in1 ? 0.0 : (out ? -1.0 : 1.0 / 15.0);
+  const double cg = out ? 1.0 : -1.0 / 15.0, cp = in1 ? 0.0 : (out ? -1.0 : 1.0 / 15.0);
+  const double r3 = in1 ? 0.0 : ri3;
   const double gp = ::fma(qq, ::fma(qq, ::fma(qq, g3, g2), g1), g0);
   const double pp = ::fma(qq * qq, ::fma(qq, ::fma(qq, ::fma(qq, p5, p4), p3), p2), p0);
-  g = ::fma(hv3, gp, ::fma(cg, ri3, g));
+  g = ::fma(hv3, gp, ::fma(cg, r3, g));
   phi = ::fma(hv, pp, ::fma(cp, ri, phi));
 }
 

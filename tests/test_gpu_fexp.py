@@ -78,7 +78,8 @@ def test_softened_pairs(n, leaf, opts, scale, shift):
     _check(pos, m, scale * r.uniform(0.05, 0.6, n), leaf, (960 + n) * U, **opts)
 
 
-@pytest.mark.parametrize("what", ["small h", "some small h", "masses", "far from the origin", "on the axes", "huge"])
+@pytest.mark.parametrize("what", ["small h", "some small h", "masses", "far from the origin", "on the axes", "huge", "close pair",
+                                  "close pair, tiny box"])
 def test_limits(what):
     n = 200
     pos, m, r = _set(n, 77)
@@ -94,6 +95,12 @@ def test_limits(what):
     elif what == "on the axes":
         pos[::3, 0] *= 1e-12
         pos[1::3, 1] = 0.0
+    elif what.startswith("close pair"):
+        # distinct particles with 1/r^3 beyond the largest double, well inside
+        # their kernels: r = 1e-110 in a box of 1, 1e-104 in one of 1e-90
+        s, r12 = (1e-90, 1e-104) if "tiny" in what else (1.0, 1e-110)
+        pos, h = pos * s, h * s
+        pos[0], pos[1] = 0.0, (r12, 0.0, 0.0)
     else:
         pos, h = pos * 1e95, h * 1e95
     _check(pos, m, h, 8, (960 + n) * U)
