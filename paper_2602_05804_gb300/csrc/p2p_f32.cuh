@@ -8,19 +8,32 @@
 // the candidates, 24 % of the pairs on a Plummer sphere) and those that cannot.
 // Both are staged in pairs and evaluated unsoftened, two sources per lane step
 // in the packed FP32 instructions; a candidate pair inside a kernel (4 % of
-// all pairs) is left out there and marked in the lane's bit masks.  The marked
-// pairs of all lanes, in lane order, are then evaluated one per lane (the
-// k-th lane finds the owner of the k-th mark and the mark in its masks), and
-// the owners add their results in order.
+// all pairs) is left out there and marked in the lane's bit masks.  Each lane
+// then evaluates its own marked pairs with both kernels.  Where one lane has
+// far more marks than the others, the marks of all lanes are dealt one per
+// lane instead, in lane order (the k-th lane finds the owner of the k-th mark
+// and the mark in its masks), and the owners add their results in order.
 //
-// Bound: instruction issue.  With the M4 kernels evaluated in place, the whole
-// warp ran them for almost every candidate step, because some lane nearly
-// always is inside a kernel: the candidates took 122 issue cycles per 32 pairs
-// where the unsoftened sources take 23.  Measured, before and now: 2.25 and
-// 1.97 ms for the 1.38e9 pairs of a Plummer sphere of 10^6 (0.80 of the issue
-// slots, 26 of 32 lanes), 7.58 and 6.48 ms at theta 0.3, 34.5 and 30.2 ms for
-// a clustered cloud of 1.6e7.
+// Bound: instruction issue.  With the M4 kernels evaluated in place for every
+// candidate, the whole warp ran them for almost every step, because some lane
+// nearly always is inside a kernel: the candidates took 122 issue cycles per
+// 32 pairs where the unsoftened sources take 23.  Measured, in place and now:
+// 2.25 and 1.86 ms for the 1.38e9 pairs of a Plummer sphere of 10^6, 7.58 and
+// 6.37 ms at theta 0.3, 34.5 and 28.4 ms for a clustered cloud of 1.6e7.
 #define P2P_RES 64  // marked pairs evaluated before their owners collect
+// A group of 32 dealt marks takes about twelve times a mark evaluated by its
+// own lane takes from a warp's lane share: own marks where the fullest lane
+// holds at most 1/12 of all (10^6 particles: 1.87 ms; 1/4 1.89, 1/8 1.88, 1/16
+// 1.90, own marks always 1.89, dealt always 1.98).
+#define P2P_OWN 12
+// Where 2 h_max of the leaf is beyond three times its size, about half of the
+// candidates lie inside a kernel and all of them are evaluated with both
+// kernels at once, without the unsoftened pass (uniform set of 3 10^5 with h of
+// 2, 3, 4, 6, 12 mean spacings, this line, never, and always the dealt marks:
+// 1.00 1.01 1.24, 2.25 2.49 3.46, 4.12 4.83 7.45, 10.1 12.7 22.0, 50.6 68.1 137
+// ms; line at 2: 10^5 particles at order 4 0.377 instead of 0.341 ms, at 4 the
+// 3-spacing set 2.39, at 6 2.48 ms).
+#define P2P_DENSE 3.0f
 struct P2PWarp {
   float4 far[P2P_SB];   // pairs, negated: [q/2] {x0, x1, y0, y1}, [SB/2 + q/2] {z0, z1, m0, m1}
   float4 near[P2P_SB];  // candidates, the same
@@ -76,6 +89,7 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
     const float4 hiL = a.geo_hi[L], loL = a.geo_lo[L];
     float lL = hiL.w * 1.0001f;
     const float hL = loL.w * 1.0001f;
+    const bool dense = 2.0f * hL > P2P_DENSE * lL;
     // lane -> (target slot, phase); more than 32 targets: a second slot, 32 on
     const int nph = (nL <= 16) ? (32 / nL) : 1;
     const int ntl = (nL <= 32) ? nL : 32;
@@ -235,8 +249,34 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
                       make_float2(d.z, d.w), fx, fy, fz, fp);
           }
         }
+        // pair of target t and candidate j with both kernels evaluated
+        auto softened = [&](int t, int j) {
+          const float4 T4 = w.tgt[t];
+          const float* const xy = reinterpret_cast<const float*>(w.near + (j >> 1)) + (j & 1);
+          const float* const zm = xy + 4 * (SB / 2);
+          const float dx = T4.x + xy[0], dy = T4.y + xy[2], dz = T4.z + zm[0];
+          const bool self = w.nloc[j] == t + 32 * slot;
+          const float nm = 0.5f * zm[2];  // -m/2
+          const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+          const float ri = (r2 > 0.0f) ? rsqrtf(r2) : 0.0f;
+          // (0 for coincident particles, no number where r^2 overflows)
+          const float r = fmaxf(fminf(r2 * ri, FLT_MAX), FLT_MIN), hj = w.nhinv[j];
+          float gi, pi, gj, pj;
+          m4_kernel<float>(r * T4.w, T4.w, ri, gi, pi);
+          m4_kernel<float>(r * hj, hj, ri, gj, pj);
+          const float mg = self ? 0.0f : nm * (gi + gj), mp = self ? 0.0f : -nm * (pi + pj);
+          return make_float4(mg * dx, mg * dy, mg * dz, mp);
+        };
+        auto take = [&](const float4& v) {
+          ax += v.x;
+          ay += v.y;
+          az += v.z;
+          pt += v.w;
+        };
+        if (dense && do_near && lane_on)
+          for (int j = ph; j < nnear; j += nph) take(softened(t0, j));
         // candidates, up to 32 steps of every lane at a time
-        for (int s0 = 0; s0 < npn; s0 += 32 * nph) {
+        for (int s0 = dense ? npn : 0; s0 < npn; s0 += 32 * nph) {
           const int end = min(npn, s0 + 32 * nph);
           unsigned m0 = 0u, m1 = 0u;  // marks of even / odd sources, the last step in bit 0
           int steps = 0;
@@ -264,6 +304,17 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
           }
           if (t0 + 32 * slot >= nL) m0 = m1 = 0u;
           const int c = __popc(m0) + __popc(m1);
+          if (__reduce_max_sync(SFMM_FULL, c) * P2P_OWN <= __reduce_add_sync(SFMM_FULL, c)) {
+            for (int k = 0; k < c; ++k) {
+              const bool odd = m0 == 0u;
+              const unsigned m = odd ? m1 : m0;
+              const int bit = 31 - __clz(m);
+              if (odd) m1 = m ^ (1u << bit);
+              else m0 = m ^ (1u << bit);
+              take(softened(t0, 2 * (s0 + ph + (steps - 1 - bit) * nph) + (odd ? 1 : 0)));
+            }
+            continue;
+          }
           int incl = c;
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
@@ -289,31 +340,11 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
                 const int c0 = __popc(om0);
                 const bool odd = rank >= c0;
                 const int bit = nth_bit(odd ? om1 : om0, odd ? rank - c0 : rank);
-                const int j = 2 * (s0 + oph + (osteps - 1 - bit) * nph) + (odd ? 1 : 0);
-                const float4 T4 = w.tgt[t];
-                const float* const xy = reinterpret_cast<const float*>(w.near + (j >> 1)) + (j & 1);
-                const float* const zm = xy + 4 * (SB / 2);
-                const float dx = T4.x + xy[0], dy = T4.y + xy[2], dz = T4.z + zm[0];
-                const bool self = w.nloc[j] == t + 32 * slot;
-                const float nm = 0.5f * zm[2];  // -m/2
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                const float ri = (r2 > 0.0f) ? rsqrtf(r2) : 0.0f;
-                const float r = (r2 > 0.0f) ? r2 * ri : FLT_MIN, hj = w.nhinv[j];
-                float gi, pi, gj, pj;
-                m4_kernel<float>(r * T4.w, T4.w, ri, gi, pi);
-                m4_kernel<float>(r * hj, hj, ri, gj, pj);
-                const float mg = self ? 0.0f : nm * (gi + gj), mp = self ? 0.0f : -nm * (pi + pj);
-                w.res[k - r0] = make_float4(mg * dx, mg * dy, mg * dz, mp);
+                w.res[k - r0] = softened(t, 2 * (s0 + oph + (osteps - 1 - bit) * nph) + (odd ? 1 : 0));
               }
             }
             __syncwarp();
-            for (int k = max(own0, r0); k < mine; ++k) {
-              const float4 v = w.res[k - r0];
-              ax += v.x;
-              ay += v.y;
-              az += v.z;
-              pt += v.w;
-            }
+            for (int k = max(own0, r0); k < mine; ++k) take(w.res[k - r0]);
             __syncwarp();
           }
         }
