@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
     const int L = a.leaf_node[leaf];
     const int fL = a.nfirst[L], nL = a.ncount[L];
     const float4 hiL = a.geo_hi[L], loL = a.geo_lo[L];
-    float lL = hiL.w * 1.0001f;
+    const float lL = hiL.w * 1.0001f;
     const float hL = loL.w * 1.0001f;
     const bool dense = 2.0f * hL > P2P_DENSE * lL;
     // lane -> (target slot, phase); more than 32 targets: a second slot, 32 on
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
       if (t < nL) {
         const float4 p = a.prel[fL + t];
         const float4 hr = a.phh[fL + t];
-        w.tgt[lane] = make_float4(p.x, p.y, p.z, hr.y < FLT_MIN ? INFINITY : hr.x);
+        w.tgt[lane] = make_float4(p.x, p.y, p.z, hr.x);
       }
       x = y = z = h2 = 0.0f;
       if (lane_on && t0 + 32 * slot < nL) {
@@ -111,18 +111,10 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
         y = p.y;
         z = p.z;
         h2 = a.phh[fL + t0 + 32 * slot].y;
-        if (h2 < FLT_MIN) h2 = INFINITY;
       }
     };
     float xi, yi, zi, h2i;
     load_targets(0, xi, yi, zi, h2i);
-    // the unsoftened loops take r^2 >= (2 h_i)^2 to be a normal number (their
-    // reciprocal square root flushes others): a leaf with a smaller h (as good
-    // as none) leaves every pair to the marked ones, where 1/h = infinity
-    // selects Newton's force at any r
-    for (int t = lane; t < nL; t += 32)
-      if (a.phh[fL + t].y < FLT_MIN) lL = INFINITY;
-    if (__any_sync(SFMM_FULL, lL == INFINITY)) lL = INFINITY;
     float ax = 0.0f, ay = 0.0f, az = 0.0f, pt = 0.0f;      // current slot
     float bx = 0.0f, by = 0.0f, bz = 0.0f, bp = 0.0f;      // the other one
 
@@ -203,7 +195,7 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
           zm[2] = v.w;
           if (near) {
             w.nh2[q] = hr.y;
-            w.nhinv[q] = hr.y < FLT_MIN ? INFINITY : hr.x;
+            w.nhinv[q] = hr.x;
             w.nloc[q] = (short)((i >= fL && i < fL + nL) ? i - fL : -1);
           }
         }
@@ -228,7 +220,7 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
           xy[3] = xy[2];
           zm[1] = zm[0];
           zm[3] = 0.0f;
-          if (lane) w.nh2[n] = 0.0f;
+          if (lane) w.nh2[n] = FLT_MIN;
         }
       }
       __syncwarp();

@@ -93,7 +93,7 @@ struct sfmm_ctx {
   DevBuf perm;                  // int32 sorted position -> input index
   DevBuf pnode;                 // int32 sorted position -> leaf node
   DevBuf prel;                  // float4 {x - s_leaf, y - s_leaf, z - s_leaf, m}
-  DevBuf phh;                   // float4 {1/h, (2h)^2, 2h rounded up, 0}
+  DevBuf phh;                   // float4 {1/h, (2h)^2, 2h rounded up, 0}, h as good as none: {inf, FLT_MIN, 1.2e-19, 0}
 
   // nodes (pre-order)
   DevBuf nfirst, ncount, nright, nparent, ndepth;

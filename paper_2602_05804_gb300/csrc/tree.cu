@@ -712,10 +712,14 @@ __global__ void __launch_bounds__(RS_NT, 4) k_rs_onesweep(const uint64_t* __rest
 // FP32 roundings of the exact values: the FP32 form's M4 kernels and its
 // inside-the-kernel test take them as they are); 2h rounded up from the
 // FP64 value, since the near-field candidate test needs a bound.
+// Where (2h)^2 is no normal number h is as good as none: 1/h = infinity, which
+// selects Newton's force at any r.  The least (2h)^2 and 2h kept still tell
+// the pairs of subnormal r^2, which the unsoftened loops do not take.
 __device__ __forceinline__ float4 softening_record(double h) {
   const float hf = __double2float_rn(h);
-  const float h2 = 2.0f * hf;
-  return make_float4(__frcp_rn(hf), h2 * h2, __double2float_ru(2.0 * h), 0.0f);
+  const float h2 = 2.0f * hf, q = h2 * h2;
+  return make_float4(q < FLT_MIN ? INFINITY : __frcp_rn(hf), fmaxf(q, FLT_MIN),
+                     fmaxf(__double2float_ru(2.0 * h), 1.2e-19f), 0.0f);
 }
 
 // Sorted particles (and their softening records, formed while the gather

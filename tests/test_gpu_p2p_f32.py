@@ -79,3 +79,9 @@ def test_kernels_beyond_the_leaves_cost_two_evaluations_a_pair():
     # a softened pair takes about 3 times an unsoftened one (6.5 times when each
     # was evaluated unsoftened, marked, dealt to a lane and handed back)
     assert _per_pair(0.2) <= 4.0 * _per_pair(1e-4)
+
+
+def test_softening_as_good_as_none_costs_no_more():
+    # every pair takes the unsoftened loops, whether (2h)^2 is a normal FP32
+    # number or not (11 times the time when every pair was a marked one)
+    assert _per_pair(1e-25) <= 1.5 * _per_pair(1e-4)
