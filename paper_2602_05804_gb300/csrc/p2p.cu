@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(P64_NT, 1) k_p2p_fp64(const P2PArgs a) {
   const unsigned lt = lanemask_lt();
   const int nextra = (int)a.d_split[0];
   const int nitems = a.items[-4];
+  if (nitems == 0) return;
   unsigned long long pairs = 0;  // this lane's share of the pair evaluations
   while (true) {
     int item = 0;
@@ -748,8 +749,10 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   if (f32) {
     k_p2p_f32<<<nblocks, P2P_NT, P2P_WARPS * sizeof(P2PWarp), c->stream>>>(a);
   } else {
-    // FP32-pipe expansions first; what they cannot take (usually nothing)
-    // is left to the FP64 kernel
+    // FP32-pipe expansions first; what they cannot take (nothing on sets near
+    // the origin with h of the order of the spacing) is left to the FP64
+    // kernel, on as many blocks as fit: with one per SM, 10^6 particles 10^7
+    // from the origin took 77.0 ms instead of 66.9
     const size_t n = (size_t)c->n;
     if ((rc = c->fx_rec.ensure((3 * sizeof(float4) + sizeof(float2) + sizeof(double2)) * n + 16)) ||
         (rc = c->fx_items.ensure(sizeof(int) * (4 + (size_t)nl_b + (size_t)nextra))))
@@ -770,7 +773,10 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
     k_p2p_fexp<<<nblocks, FX_NT, 0, c->stream>>>(a, f);
     a.leaf_counter = f.fb + 1;
     a.items = f.fb + 4;
-    k_p2p_fp64<<<num_sms(c->device), P64_NT, 0, c->stream>>>(a);
+    int fit64 = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit64, k_p2p_fp64, P64_NT, 0);
+    if (c->p2p_blocks > 0 && c->p2p_blocks < fit64) fit64 = c->p2p_blocks;
+    k_p2p_fp64<<<std::max(1, fit64) * num_sms(c->device), P64_NT, 0, c->stream>>>(a);
     c->nlaunch += 2;
   }
   ++c->nlaunch;

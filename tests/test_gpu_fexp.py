@@ -122,3 +122,24 @@ def test_systems_of_different_scales():
         ra, rp, A, B = _direct(pos[a:b], m[a:b], h[a:b])
         assert (np.abs(acc[a:b] - ra) <= (960 + b - a) * U * A + 1e-300).all()
         assert (np.abs(pot[a:b] - rp) <= (960 + b - a) * U * B + 1e-300).all()
+
+
+def _near_field_ms(pos, m, h, **opts):
+    s = solver("fp64", profile=1, **opts)
+    s.build(pos, m, h, 16)
+    best = np.inf
+    for _ in range(5):
+        s.gravity(0.5, 2)
+        best = min(best, s.stats()["ms_p2p"])
+    s.close()
+    return best
+
+
+def test_items_left_to_fp64_fill_the_gpu():
+    # far from the origin every item is left to the FP64 kernel: three blocks
+    # per SM against one (0.86 of its time; equal while one was all it got)
+    import workloads
+
+    pos, m, h = workloads.plummer(100_000, 31)
+    pos = pos + 1e7
+    assert _near_field_ms(pos, m, h) <= 0.95 * _near_field_ms(pos, m, h, p2p_blocks=1)
