@@ -129,8 +129,11 @@ int sfmm_set_stream(sfmm_ctx* ctx, void* stream);
  *                    lists are cut into chunks evaluated as separate items
  *                    and recombined in chunk order (default 256, 32..65536;
  *                    fewer are taken, down to 8, when all lists together are
- *                    too short to occupy the GPU)
- *   "p2p_blocks"     near-field blocks per SM (0, default: as many as fit)
+ *                    too short to occupy the GPU: the order of a sum, and with
+ *                    it the last bits of a result, then depend on the length
+ *                    of all lists of the call and on the device)
+ *   "p2p_blocks"     near-field blocks per SM (0, default: as many as fit);
+ *                    bitwise the same results
  *   "autotune_theta", "autotune_order"  theta and order that autotuned leaf
  *                    sizes are chosen for (sfmm_build_batch with NULL sizes)
  *   "profile"        1 records per-stage device times into the stats

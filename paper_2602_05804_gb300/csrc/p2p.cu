@@ -73,7 +73,7 @@ struct P2PArgs {
 // entries throughout, the near field of 1000 particles took 54 us in 96 items
 // and that of 13,000 in the FP64 form 4.9 ms in 2500 items on 2432 warps; 32 us
 // and 2.0 ms now.
-__host__ __device__ __forceinline__ int p2p_chunk_of(unsigned long long total, int most, int want) {
+__device__ __forceinline__ int p2p_chunk_of(unsigned long long total, int most, int want) {
   const unsigned long long c = total / (unsigned)want;
   return c >= (unsigned long long)most ? most : (c < 8 ? 8 : (int)c);
 }
@@ -683,7 +683,8 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   const int fit = p2p_blocks_fit(c);
   const int per_sm = (c->p2p_blocks > 0 && c->p2p_blocks < fit) ? c->p2p_blocks : fit;  // option: fewer
   const int nblocks = per_sm * num_sms(c->device);
-  const int want = 8 * nblocks * (f32 ? P2P_WARPS : FX_WARPS);
+  // (from the blocks that fit: the option changes no sum's order)
+  const int want = 8 * fit * num_sms(c->device) * (f32 ? P2P_WARPS : FX_WARPS);
   // long lists: slots, extra items and split leaves are counted by the split
   // pass on the device; the buffers are sized from bounds on the host (a list
   // of cnt > chunk entries takes ceil(cnt / chunk) <= 2 cnt / chunk slots, and

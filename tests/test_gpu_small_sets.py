@@ -81,6 +81,22 @@ def test_few_lists_are_cut_finer(prec, n, leaf):
         assert acc_rel(acc, a_o).max() <= tol and pot_rel(pot, p_o).max() <= tol
 
 
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("n", [700, 5000])
+def test_blocks_per_sm_change_no_bit(prec, n):
+    # where the lists are cut depends on the blocks that fit, not on those taken
+    pos, m, h = workloads.plummer(n, 12)
+    got = []
+    for blocks in (0, 1, 2):
+        s = solver(prec, p2p_blocks=blocks)
+        s.build(pos, m, h, 16)
+        got.append([t.cpu().numpy() for t in s.gravity(0.5, 2)])
+        s.close()
+    for a, p in got[1:]:
+        np.testing.assert_array_equal(a, got[0][0])
+        np.testing.assert_array_equal(p, got[0][1])
+
+
 @pytest.mark.parametrize("order", [1, 2, 3, 4])
 @pytest.mark.parametrize("n,leaf", [(2, 1), (5, 1), (40, 1), (300, 2), (3000, 1), (20000, 16)])
 def test_moments_of_the_climb(order, n, leaf):
