@@ -73,9 +73,10 @@ struct P2PArgs {
 // entries throughout, the near field of 1000 particles took 54 us in 96 items
 // and that of 13,000 in the FP64 form 4.9 ms in 2500 items on 2432 warps; 32 us
 // and 2.0 ms now.
+#define P2P_CHUNK_LEAST 8
 __device__ __forceinline__ int p2p_chunk_of(unsigned long long total, int most, int want) {
   const unsigned long long c = total / (unsigned)want;
-  return c >= (unsigned long long)most ? most : (c < 8 ? 8 : (int)c);
+  return c >= (unsigned long long)most ? most : (c < P2P_CHUNK_LEAST ? P2P_CHUNK_LEAST : (int)c);
 }
 
 // M4 softening kernel of one particle (compact support 2h): g = phi'(r)/r
@@ -686,21 +687,21 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   // (from the blocks that fit: the option changes no sum's order)
   const int want = 8 * fit * num_sms(c->device) * (f32 ? P2P_WARPS : FX_WARPS);
   // long lists: slots, extra items and split leaves are counted by the split
-  // pass on the device; the buffers are sized from bounds on the host (a list
-  // of cnt > chunk entries takes ceil(cnt / chunk) <= 2 cnt / chunk slots, and
-  // entries / chunk is at most arena / maximum or 9/8 want), with no wait for
-  // the walk
+  // pass on the device; the buffers are sized from bounds on the host, with no
+  // wait for the walk: E entries in all (at most the arena's) in chunks of C
+  // give at most E / C slots and one more per split list, of which there are at
+  // most E / C too; E / C is at most arena / maximum or want + want / least
+  // (the rounding of C), and arena / least in any case
   const int most = c->p2p_chunk;
+  const int nl_b = c->graph_mode ? (int)c->n : nl;  // leaf-indexed: the bound for a captured step
   const int64_t arena_cap = (int64_t)(c->arena.bytes / sizeof(int));
-  const int nslots =
-      (int)std::min<int64_t>(std::max<int64_t>(2 * arena_cap / most, 3 * (int64_t)want) + 2, INT32_MAX / 2);
-  const int nsplit = (int)std::min<int64_t>(
-      std::min<int64_t>(c->graph_mode ? c->n : nl, std::max<int64_t>(arena_cap / (most + 1), 2 * (int64_t)want) + 1),
-      nslots);
+  const int64_t full = std::min<int64_t>(
+      arena_cap / P2P_CHUNK_LEAST + 1, std::max<int64_t>(arena_cap / most, (int64_t)want + want / P2P_CHUNK_LEAST) + 1);
+  const int nsplit = (int)std::min<int64_t>(nl_b, full);
+  const int nslots = (int)std::min<int64_t>(full + nsplit, INT32_MAX / 2);
   const int nextra = nslots;
   int lmax = c->leaf_size;
   for (int v : c->h_sys_lsz) lmax = v > lmax ? v : lmax;
-  const int nl_b = c->graph_mode ? (int)c->n : nl;  // leaf-indexed: the bound for a captured step
   if ((rc = c->p2p_split.ensure(sizeof(int) * (size_t)nl_b))) return rc;
   if ((rc = c->p2p_extra.ensure(sizeof(int2) * (size_t)nextra))) return rc;
   if ((rc = c->p2p_slist.ensure(sizeof(int) * (size_t)nsplit))) return rc;

@@ -97,6 +97,26 @@ def test_blocks_per_sm_change_no_bit(prec, n):
         np.testing.assert_array_equal(p, got[0][1])
 
 
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_device_memory_of_small_sets(prec):
+    # partial sums of cut lists are bounded by what the set's lists can hold: at
+    # most a MB or two for 1000 particles (a bound by the GPU's size alone was
+    # 120 MB more with leaves of 64 than a leaf size that cuts no list takes)
+    import torch
+
+    taken = []
+    for leaf in (16, 64):
+        pos, m, h = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in workloads.plummer(1000, 4))
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        s = solver(prec)
+        s.build(pos, m, h, leaf)
+        s.gravity(0.5, 2)
+        taken.append(free - torch.cuda.mem_get_info()[0])
+        s.close()
+    assert abs(taken[1] - taken[0]) <= 16 << 20
+
+
 @pytest.mark.parametrize("order", [1, 2, 3, 4])
 @pytest.mark.parametrize("n,leaf", [(2, 1), (5, 1), (40, 1), (300, 2), (3000, 1), (20000, 16)])
 def test_moments_of_the_climb(order, n, leaf):
