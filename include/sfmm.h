@@ -128,10 +128,11 @@ int sfmm_set_stream(sfmm_ctx* ctx, void* stream);
  *   "p2p_chunk"      neighbour-list entries per near-field work item: longer
  *                    lists are cut into chunks evaluated as separate items
  *                    and recombined in chunk order (default 256, 32..65536;
- *                    fewer are taken, down to 8, when all lists together are
- *                    too short to occupy the GPU: the order of a sum, and with
- *                    it the last bits of a result, then depend on the length
- *                    of all lists of the call and on the device)
+ *                    fewer are taken, down to 8 (256 at leaf size 1), when
+ *                    all lists together are too short to occupy the GPU: the
+ *                    order of a sum, and with it the last bits of a result,
+ *                    then depend on the length of all lists of the call and on
+ *                    the device)
  *   "p2p_blocks"     near-field blocks per SM (0, default: as many as fit);
  *                    bitwise the same results
  *   "autotune_theta", "autotune_order"  theta and order that autotuned leaf

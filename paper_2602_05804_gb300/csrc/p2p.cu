@@ -68,15 +68,24 @@ struct P2PArgs {
 };
 
 // Neighbour-list entries per work item: the option's value, fewer when the
-// lists are too few for eight items per resident warp, down to 8 entries (an
-// item then stages about a warp's width of sources a few times).  With 256
-// entries throughout, the near field of 1000 particles took 54 us in 96 items
-// and that of 13,000 in the FP64 form 4.9 ms in 2500 items on 2432 warps; 32 us
-// and 2.0 ms now.
-#define P2P_CHUNK_LEAST 8
-__device__ __forceinline__ int p2p_chunk_of(unsigned long long total, int most, int want) {
+// lists are too few for eight items per resident warp, down to p2p_chunk_least.
+// With 256 entries throughout, the near field of 1000 particles took 54 us in
+// 96 items and that of a binary of 13,000 in the FP64 form (several calls of a
+// leapfrog run) 4.9 ms in 2500 items on 2432 warps; 32 us and 2.0 ms cut finer.
+__device__ __forceinline__ int p2p_chunk_of(unsigned long long total, int most, int least, int want) {
   const unsigned long long c = total / (unsigned)want;
-  return c >= (unsigned long long)most ? most : (c < P2P_CHUNK_LEAST ? P2P_CHUNK_LEAST : (int)c);
+  return c >= (unsigned long long)most ? most : max(least, (int)c);
+}
+
+// The least: 8 entries, more where leaves are so small that 8 of them hold too
+// few pairs for an item's fixed costs (its start, its partial sums and their
+// addition).  Pairs of full leaves that pay for an item: 1024 in the FP32 form
+// (binary of 5000 with leaves of 1, 4 and 8 particles: 42, 37 and 46 us instead
+// of 97, 75 and 53 with 8 entries; Plummer spheres of 300 to 500 are within 3 us
+// of it, where 2048 costs up to 8), 128 in the FP64 form, whose pairs take
+// longer (2000 particles with leaves of 1: 155 us instead of 236; 512: 175).
+static int p2p_chunk_least(bool f32, int leaf, int most) {
+  return std::min(most, std::max(8, (f32 ? 1024 : 128) / (leaf * leaf)));
 }
 
 // M4 softening kernel of one particle (compact support 2h): g = phi'(r)/r
@@ -583,9 +592,10 @@ __global__ void __launch_bounds__(P64_NT, 1) k_p2p_fp64(const P2PArgs a) {
 __global__ void k_p2p_split(const uint32_t* __restrict__ counts, const int* __restrict__ p2p_cnt,
                             int* __restrict__ split, int2* __restrict__ extra, int* __restrict__ slist,
                             unsigned long long* __restrict__ ctr, int max_extra, int max_slots, int max_split,
-                            int most, int want, const unsigned long long* __restrict__ list_total,
+                            int most, int least, int want,
+                            const unsigned long long* __restrict__ list_total,
                             unsigned long long* __restrict__ chunk_now, int* __restrict__ status) {
-  const int chunk = p2p_chunk_of(*list_total, most, want);
+  const int chunk = p2p_chunk_of(*list_total, most, least, want);
   if (blockIdx.x == 0 && threadIdx.x == 0) *chunk_now = (unsigned long long)chunk;
   const int nleaves = (int)counts[1];
   const int lane = threadIdx.x & 31;
@@ -686,22 +696,23 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   const int nblocks = per_sm * num_sms(c->device);
   // (from the blocks that fit: the option changes no sum's order)
   const int want = 8 * fit * num_sms(c->device) * (f32 ? P2P_WARPS : FX_WARPS);
+  int lmax = c->leaf_size;
+  for (int v : c->h_sys_lsz) lmax = v > lmax ? v : lmax;
+  const int most = c->p2p_chunk;
+  const int least = p2p_chunk_least(f32, lmax, most);
   // long lists: slots, extra items and split leaves are counted by the split
   // pass on the device; the buffers are sized from bounds on the host, with no
   // wait for the walk: E entries in all (at most the arena's) in chunks of C
   // give at most E / C slots and one more per split list, of which there are at
   // most E / C too; E / C is at most arena / maximum or want + want / least
   // (the rounding of C), and arena / least in any case
-  const int most = c->p2p_chunk;
   const int nl_b = c->graph_mode ? (int)c->n : nl;  // leaf-indexed: the bound for a captured step
   const int64_t arena_cap = (int64_t)(c->arena.bytes / sizeof(int));
   const int64_t full = std::min<int64_t>(
-      arena_cap / P2P_CHUNK_LEAST + 1, std::max<int64_t>(arena_cap / most, (int64_t)want + want / P2P_CHUNK_LEAST) + 1);
+      arena_cap / least + 1, std::max<int64_t>(arena_cap / most, (int64_t)want + want / least) + 1);
   const int nsplit = (int)std::min<int64_t>(nl_b, full);
   const int nslots = (int)std::min<int64_t>(full + nsplit, INT32_MAX / 2);
   const int nextra = nslots;
-  int lmax = c->leaf_size;
-  for (int v : c->h_sys_lsz) lmax = v > lmax ? v : lmax;
   if ((rc = c->p2p_split.ensure(sizeof(int) * (size_t)nl_b))) return rc;
   if ((rc = c->p2p_extra.ensure(sizeof(int2) * (size_t)nextra))) return rc;
   if ((rc = c->p2p_slist.ensure(sizeof(int) * (size_t)nsplit))) return rc;
@@ -709,7 +720,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
   const int sblocks = std::max(1, std::min((nl_b + 255) / 256, 8 * num_sms(c->device)));
   k_p2p_split<<<sblocks, 256, 0, c->stream>>>(c->d_counts, c->p2p_cnt.as<int>(), c->p2p_split.as<int>(),
                                                      c->p2p_extra.as<int2>(), c->p2p_slist.as<int>(), ctr + 11,
-                                                     nextra, nslots, nsplit, most, want, ctr + 9, ctr + 7, c->d_status);
+                                                     nextra, nslots, nsplit, most, least, want, ctr + 9, ctr + 7, c->d_status);
   ++c->nlaunch;
   SFMM_CUDA_TRY(cudaGetLastError());
   P2PArgs a{};

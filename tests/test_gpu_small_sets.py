@@ -68,7 +68,7 @@ def test_sums_of_sliced_systems():
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-@pytest.mark.parametrize("n,leaf", [(60, 4), (700, 16), (700, 64), (5000, 33)])
+@pytest.mark.parametrize("n,leaf", [(60, 4), (700, 16), (700, 64), (5000, 33), (3000, 1), (3000, 2), (2500, 7)])
 def test_few_lists_are_cut_finer(prec, n, leaf):
     pos, m, h = workloads.binary_polytrope(n, 9)
     a_o, p_o, _ = oracle.sfmm(pos, m, h, theta=0.4, p=2, leaf_size=leaf)
@@ -79,6 +79,23 @@ def test_few_lists_are_cut_finer(prec, n, leaf):
         acc, pot = (t.cpu().numpy() for t in s.gravity(0.4, 2))
         s.close()
         assert acc_rel(acc, a_o).max() <= tol and pot_rel(pot, p_o).max() <= tol
+
+
+def test_leaves_of_one_are_not_cut_into_crumbs():
+    # an item of 8 one-particle leaves costs its start and end: twice the time
+    # of leaves of 16 (0.9 of it with 256 entries)
+    pos, m, h = workloads.binary_polytrope(5000, 9)
+    ms = []
+    for leaf in (1, 16):
+        s = solver("fp32", profile=1)
+        s.build(pos, m, h, leaf)
+        best = np.inf
+        for _ in range(8):
+            s.gravity(0.5, 2)
+            best = min(best, s.stats()["ms_p2p"])
+        ms.append(best)
+        s.close()
+    assert ms[0] <= 1.3 * ms[1], ms
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
