@@ -23,15 +23,18 @@ namespace sfmm {
 
 // Tree over the threads' sums: one (pair of threads, sum) per thread and
 // trip, so that the narrow FP64 pipe runs full warps (a thread merging all
-// five sums of its pair took 12 us for a set of 1000 particles).
-__device__ __forceinline__ void block_merge(csum (&s)[5], double (&sh)[10][RED_NT]) {
+// five sums of its pair took 12 us for a set of 1000 particles).  used: threads
+// that hold a sum (the tree of a system of ten particles needs no 256 of them).
+__device__ __forceinline__ void block_merge(csum (&s)[5], double (&sh)[10][RED_NT], int used = RED_NT) {
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     sh[c][threadIdx.x] = s[c].s;
     sh[5 + c][threadIdx.x] = s[c].c;
   }
   __syncthreads();
-  for (int w = RED_NT / 2; w > 0; w >>= 1) {
+  int top = RED_NT / 2;
+  while (top > 0 && top >= used) top >>= 1;
+  for (int w = top; w > 0; w >>= 1) {
     for (int q = threadIdx.x; q < 5 * w; q += RED_NT) {
       const int c = q / w, t = q - c * w;
       csum a{sh[c][t], sh[5 + c][t]};
@@ -75,46 +78,60 @@ __global__ void __launch_bounds__(RED_NT) k_reduce_particles(int64_t n, const do
   if (threadIdx.x < 10) part[10 * blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
 }
 
-// One warp per sum (block c: sum c), on five SMs: lane l merges partials l,
-// l + 32, ... in order, then the lanes merge in a fixed tree.
-__global__ void k_reduce_final(int nparts, const double* __restrict__ part, double* __restrict__ out) {
+// One warp per sum (block c: sum c): lane l merges partials lo + l, lo + l +
+// 32, ... in order, then the lanes merge in a fixed tree (lane 0 holds it).
+__device__ __forceinline__ csum merge_parts(int lo, int hi, const double* __restrict__ part) {
   const int c = blockIdx.x, lane = threadIdx.x;
   csum s{0.0, 0.0};
-  for (int q = lane; q < nparts; q += 32) cs_merge(s, part[10 * q + c], part[10 * q + 5 + c]);
+  for (int q = lo + lane; q < hi; q += 32) cs_merge(s, part[10 * q + c], part[10 * q + 5 + c]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const double bs = __shfl_down_sync(SFMM_FULL, s.s, o), bc = __shfl_down_sync(SFMM_FULL, s.c, o);
     if (lane < o) cs_merge(s, bs, bc);
   }
-  if (lane == 0) out[c] = __dadd_rn(s.s, s.c);
+  return s;
+}
+__global__ void k_reduce_final(int nparts, const double* __restrict__ part, double* __restrict__ out) {
+  const csum s = merge_parts(0, nparts, part);
+  if (threadIdx.x == 0) out[blockIdx.x] = __dadd_rn(s.s, s.c);
+}
+// Many partials: RED_GROUP of them to one first (60,000 systems left five warps
+// 1900 FP64 additions one after another).
+#define RED_GROUP 1024
+__global__ void k_reduce_group(int nparts, const double* __restrict__ part, double* __restrict__ out) {
+  const int lo = blockIdx.y * RED_GROUP;
+  const csum s = merge_parts(lo, min(nparts, lo + RED_GROUP), part);
+  if (threadIdx.x == 0) {
+    out[10 * (size_t)blockIdx.y + blockIdx.x] = s.s;
+    out[10 * (size_t)blockIdx.y + 5 + blockIdx.x] = s.c;
+  }
 }
 
-// Batches: block (k, system) takes the k-th of gridDim.x equal slices of the
-// system's sorted positions (systems are contiguous in the sorted order).
-__global__ void __launch_bounds__(RED_NT) k_reduce_slices(const int* __restrict__ sys_off,
+// Batches: a block per slice (batch_slice) of a system's sorted positions
+// (systems are contiguous in the sorted order).
+__global__ void __launch_bounds__(RED_NT) k_reduce_slices(int nsys, const int* __restrict__ sys_off, int shift,
                                                           const double* __restrict__ pm,
                                                           const int* __restrict__ perm,
                                                           const double* __restrict__ acc,
                                                           const double* __restrict__ pot, double* __restrict__ part) {
   __shared__ double sh[10][RED_NT];
-  const int sys = blockIdx.y;
-  const int64_t b = sys_off[sys], cnt = sys_off[sys + 1] - b;
+  const BatchSlice b = batch_slice(sys_off, nsys, shift, blockIdx.x);
   csum s[5] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
-  particle_sums(b + cnt * blockIdx.x / gridDim.x, b + cnt * (blockIdx.x + 1) / gridDim.x, pm, perm, acc, pot, s);
-  block_merge(s, sh);
-  if (threadIdx.x < 10) part[10 * ((size_t)sys * gridDim.x + blockIdx.x) + threadIdx.x] = sh[threadIdx.x][0];
+  particle_sums(b.lo, b.hi, pm, perm, acc, pot, s);
+  block_merge(s, sh, (int)min((int64_t)RED_NT, b.hi - b.lo));
+  if (threadIdx.x < 10) part[10 * (size_t)blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
 }
 
 // One thread per (system, sum): the slices merged in order, as the system's
 // partial (for the sums over all systems) and as its value.
-__global__ void k_reduce_sys(int nsys, int slices, const double* __restrict__ part, double* __restrict__ sys_part,
-                             double* __restrict__ out) {
+__global__ void k_reduce_sys(int nsys, const int* __restrict__ sys_off, int shift, const double* __restrict__ part,
+                             double* __restrict__ sys_part, double* __restrict__ out) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 5 * nsys) return;
   const int sys = t / 5, c = t - 5 * sys;
   csum s{0.0, 0.0};
-  for (int k = 0; k < slices; ++k) {
-    const double* q = part + 10 * ((size_t)sys * slices + k);
+  for (int k = slice_base(sys_off, shift, sys); k < slice_base(sys_off, shift, sys + 1); ++k) {
+    const double* q = part + 10 * (size_t)k;
     cs_merge(s, q[c], q[5 + c]);
   }
   sys_part[10 * (size_t)sys + c] = s.s;
@@ -124,33 +141,40 @@ __global__ void k_reduce_sys(int nsys, int slices, const double* __restrict__ pa
 }
 
 // Sums over all particles (device pointer in *out_dev) and, for batches, per
-// system.  Slices of at most 8192 particles: one block per system took 1.45 ms
-// for 256 systems of up to 10^5 particles, beside a second pass for the totals.
+// system, in slices of at most 8192 particles (of 1/64 of the largest system,
+// where that is more: one thread per system and sum adds its slices).  One block
+// per system took 1.45 ms for 256 systems of up to 10^5 particles, beside a
+// second pass for the totals; as many slices for every system as the largest
+// needs 70 ms for one of 5 10^5 among 60,000 of ten (0.5 ms now).
 int run_reduce(sfmm_ctx* c, double** out_dev) {
   int rc;
   const bool batch = c->nsys > 1;
-  int64_t largest = 0;
-  for (int k = 0; k < c->nsys; ++k) largest = std::max(largest, c->h_sys_off[k + 1] - c->h_sys_off[k]);
-  const int slices = (int)std::min<int64_t>(64, (largest + 8191) / 8192);
+  const int shift = slice_shift(c, 13, 64);
+  const size_t slices = batch ? (size_t)(c->n >> shift) + c->nsys : 0;
   const int blocks = (int)std::min<int64_t>(RED_BLOCKS, (c->n + RED_NT - 1) / RED_NT);
-  const size_t nparts = batch ? (size_t)c->nsys * (slices + 1) : (size_t)blocks;
+  const int groups = c->nsys > RED_GROUP ? (c->nsys + RED_GROUP - 1) / RED_GROUP : 0;
+  const size_t nparts = batch ? slices + c->nsys + groups : (size_t)blocks;
   if ((rc = c->red_part.ensure(sizeof(double) * 10 * (nparts + 1)))) return rc;
   double* part = c->red_part.as<double>();
   double* out = part + 10 * nparts;
   if (batch) {
     if ((rc = c->sys_sums.ensure(sizeof(double) * 5 * (size_t)c->nsys))) return rc;
-    double* sys_part = part + 10 * (size_t)c->nsys * slices;
-    for (int s0 = 0; s0 < c->nsys; s0 += 65535) {  // (the grid's y limit)
-      const int ns = std::min(65535, c->nsys - s0);
-      k_reduce_slices<<<dim3(slices, ns), RED_NT, 0, c->stream>>>(
-          c->sys_off.as<int>() + s0, c->pm.as<double>(), c->perm.as<int>(), c->red_acc, c->red_pot,
-          part + 10 * (size_t)s0 * slices);
-      ++c->nlaunch;
-    }
-    k_reduce_sys<<<(5 * c->nsys + 127) / 128, 128, 0, c->stream>>>(c->nsys, slices, part, sys_part,
+    double* sys_part = part + 10 * slices;
+    const int* off = c->sys_off.as<int>();
+    k_reduce_slices<<<(unsigned)slices, RED_NT, 0, c->stream>>>(c->nsys, off, shift, c->pm.as<double>(),
+                                                                c->perm.as<int>(), c->red_acc, c->red_pot, part);
+    ++c->nlaunch;
+    k_reduce_sys<<<(5 * c->nsys + 127) / 128, 128, 0, c->stream>>>(c->nsys, off, shift, part, sys_part,
                                                                    c->sys_sums.as<double>());
     ++c->nlaunch;
-    k_reduce_final<<<5, 32, 0, c->stream>>>(c->nsys, sys_part, out);
+    if (groups) {
+      double* grouped = sys_part + 10 * (size_t)c->nsys;
+      k_reduce_group<<<dim3(5, groups), 32, 0, c->stream>>>(c->nsys, sys_part, grouped);
+      ++c->nlaunch;
+      k_reduce_final<<<5, 32, 0, c->stream>>>(groups, grouped, out);
+    } else {
+      k_reduce_final<<<5, 32, 0, c->stream>>>(c->nsys, sys_part, out);
+    }
   } else {
     k_reduce_particles<<<blocks, RED_NT, 0, c->stream>>>(c->n, c->pm.as<double>(), c->perm.as<int>(), c->red_acc,
                                                         c->red_pot, part);

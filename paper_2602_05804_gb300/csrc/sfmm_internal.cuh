@@ -1,6 +1,7 @@
 // Internal declarations of the SFMM gravity library: the context and the
 // stage launchers implemented in tree.cu, moments.cu, walk.cu, p2p.cu.
 #pragma once
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -188,6 +189,40 @@ unsigned long long buffers_fingerprint(sfmm_ctx* c);  // their addresses and siz
 
 int check_status(sfmm_ctx* c);
 int sync_status(sfmm_ctx* c, int* bits, bool counts = false);
+
+// A batch's particles in slices, a block each: system s has the slices
+// [slice_base(s), slice_base(s + 1)), one more than the multiples of 2^shift in
+// (off[s], off[s + 1]], hence enough for slices of at most 2^shift particles,
+// and (n >> shift) + nsys in all, however the sizes are mixed.
+__device__ __forceinline__ int slice_base(const int* __restrict__ off, int shift, int s) { return (off[s] >> shift) + s; }
+struct BatchSlice {
+  int sys, first, count;  // the system, its first slice and how many it has
+  int64_t lo, hi;         // the slice's particles
+};
+__device__ __forceinline__ BatchSlice batch_slice(const int* __restrict__ off, int nsys, int shift, int k) {
+  int s = 0, e = nsys;  // the last system whose first slice is not above k
+  while (e - s > 1) {
+    const int m = (s + e) >> 1;
+    if (slice_base(off, shift, m) <= k) s = m;
+    else e = m;
+  }
+  BatchSlice b;
+  b.sys = s;
+  b.first = slice_base(off, shift, s);
+  b.count = slice_base(off, shift, s + 1) - b.first;
+  const int64_t o = off[s], n = off[s + 1] - o;
+  b.lo = o + n * (k - b.first) / b.count;
+  b.hi = o + n * (k - b.first + 1) / b.count;
+  return b;
+}
+// Slice length 2^shift: at least 2^least, and at most `most` full ones in a system.
+inline int slice_shift(const sfmm_ctx* c, int least, int most) {
+  int64_t largest = 0;
+  for (int k = 0; k < c->nsys; ++k) largest = std::max(largest, c->h_sys_off[k + 1] - c->h_sys_off[k]);
+  int shift = least;
+  while (largest >> shift > most) ++shift;
+  return shift;
+}
 
 inline int num_sms(int device) {
   int v = 0;

@@ -67,6 +67,42 @@ def test_sums_of_sliced_systems():
     assert abs(st["W"] - 0.5 * math.fsum(m * pot)) <= 1e-14 * abs(st["W"])
 
 
+def _sums_batch(sizes):
+    pos, m, h = workloads.plummer(int(sum(sizes)), 17)
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    s = solver("fp32", profile=1)
+    best = np.inf
+    for _ in range(3):
+        s.build_batch(off, pos, m, h, np.full(len(sizes), 16, np.int32))
+        acc, pot = s.gravity(0.8, 1)
+        best = min(best, s.stats()["ms_reduce"])
+    out = s.batch_sums(), s.stats(), m[:, None] * acc.cpu().numpy(), m * pot.cpu().numpy(), off, best
+    s.close()
+    return out
+
+
+def test_sums_of_one_large_system_among_small_ones():
+    # slices of 8192 particles up to 64 of them, longer beyond; 1024 systems'
+    # sums are added in a group
+    r = np.random.default_rng(3)
+    sizes = np.concatenate([r.integers(1, 12, 1500), [530_001], r.integers(1, 12, 18500)])
+    sums, st, ma, mp, off, ms = _sums_batch(sizes)
+    for k in list(range(0, len(sizes), 97)) + [1499, 1500, 1501, len(sizes) - 1]:
+        a, b = off[k], off[k + 1]
+        for c in range(3):
+            x = math.fsum(ma[a:b, c])
+            assert abs(sums[k, c] - x) <= 4e-16 * abs(x) + 1e-25 * np.abs(ma[a:b, c]).sum(), (k, c)
+        assert abs(sums[k, 3] - np.abs(ma[a:b]).sum()) <= 1e-13 * sums[k, 3]
+        assert abs(sums[k, 4] - 0.5 * mp[a:b].sum()) <= 1e-13 * np.abs(mp[a:b]).sum()
+    for c in range(3):
+        x = math.fsum(ma[:, c])
+        assert abs(st["momentum"][c] - x) <= 4e-16 * abs(x) + 1e-25 * np.abs(ma).sum()
+    assert abs(st["W"] - 0.5 * math.fsum(mp)) <= 1e-13 * abs(st["W"])
+    # no system pays for the largest one (64 slices for each: 30 times)
+    even = np.full(len(sizes), sizes.sum() // len(sizes))
+    assert ms <= 6.0 * _sums_batch(even)[-1]
+
+
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
 @pytest.mark.parametrize("n,leaf", [(60, 4), (700, 16), (700, 64), (5000, 33), (3000, 1), (3000, 2), (2500, 7)])
 def test_few_lists_are_cut_finer(prec, n, leaf):
