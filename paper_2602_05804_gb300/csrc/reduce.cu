@@ -145,7 +145,7 @@ __global__ void k_reduce_sys(int nsys, const int* __restrict__ sys_off, int shif
 // where that is more: one thread per system and sum adds its slices).  One block
 // per system took 1.45 ms for 256 systems of up to 10^5 particles, beside a
 // second pass for the totals; as many slices for every system as the largest
-// needs 70 ms for one of 5 10^5 among 60,000 of ten (0.5 ms now).
+// needs took 70 ms for one of 5 10^5 among 60,000 of ten (0.4 ms now).
 int run_reduce(sfmm_ctx* c, double** out_dev) {
   int rc;
   const bool batch = c->nsys > 1;

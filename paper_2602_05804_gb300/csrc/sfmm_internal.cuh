@@ -199,12 +199,16 @@ struct BatchSlice {
   int sys, first, count;  // the system, its first slice and how many it has
   int64_t lo, hi;         // the slice's particles
 };
+// Slice k, by whole warps: the last system whose first slice is not above k, in
+// steps of 32 (with one lane's binary search the build of 60,000 systems of ten
+// took 0.82 ms instead of 0.69).
 __device__ __forceinline__ BatchSlice batch_slice(const int* __restrict__ off, int nsys, int shift, int k) {
-  int s = 0, e = nsys;  // the last system whose first slice is not above k
+  int s = shift < 31 ? 0 : k, e = shift < 31 ? nsys : k + 1;
   while (e - s > 1) {
-    const int m = (s + e) >> 1;
-    if (slice_base(off, shift, m) <= k) s = m;
-    else e = m;
+    const int step = (e - s + 31) >> 5, m = s + (lane_id() + 1) * step;
+    const int below = __popc(__ballot_sync(SFMM_FULL, m < e && slice_base(off, shift, m) <= k));
+    s += below * step;
+    e = min(e, s + step);
   }
   BatchSlice b;
   b.sys = s;
@@ -215,10 +219,12 @@ __device__ __forceinline__ BatchSlice batch_slice(const int* __restrict__ off, i
   b.hi = o + n * (k - b.first + 1) / b.count;
   return b;
 }
-// Slice length 2^shift: at least 2^least, and at most `most` full ones in a system.
+// Slice length 2^shift: at least 2^least, and at most `most` full ones in a
+// system; 31 where none needs a second slice (slice k is system k then).
 inline int slice_shift(const sfmm_ctx* c, int least, int most) {
   int64_t largest = 0;
   for (int k = 0; k < c->nsys; ++k) largest = std::max(largest, c->h_sys_off[k + 1] - c->h_sys_off[k]);
+  if (largest <= int64_t(1) << least) return 31;
   int shift = least;
   while (largest >> shift > most) ++shift;
   return shift;

@@ -71,11 +71,11 @@ def _sums_batch(sizes):
     pos, m, h = workloads.plummer(int(sum(sizes)), 17)
     off = np.concatenate([[0], np.cumsum(sizes)])
     s = solver("fp32", profile=1)
-    best = np.inf
-    for _ in range(3):
+    best = [np.inf, np.inf]
+    for _ in range(4):
         s.build_batch(off, pos, m, h, np.full(len(sizes), 16, np.int32))
         acc, pot = s.gravity(0.8, 1)
-        best = min(best, s.stats()["ms_reduce"])
+        best = [min(best[0], s.stats()["ms_reduce"]), min(best[1], s.stats()["ms_build"])]
     out = s.batch_sums(), s.stats(), m[:, None] * acc.cpu().numpy(), m * pot.cpu().numpy(), off, best
     s.close()
     return out
@@ -98,9 +98,11 @@ def test_sums_of_one_large_system_among_small_ones():
         x = math.fsum(ma[:, c])
         assert abs(st["momentum"][c] - x) <= 4e-16 * abs(x) + 1e-25 * np.abs(ma).sum()
     assert abs(st["W"] - 0.5 * math.fsum(mp)) <= 1e-13 * abs(st["W"])
-    # no system pays for the largest one (64 slices for each: 30 times)
-    even = np.full(len(sizes), sizes.sum() // len(sizes))
-    assert ms <= 6.0 * _sums_batch(even)[-1]
+    # no system pays for the largest one (64 slices of the sums for each: 39
+    # times, and 32 of the boxes: 3.6 times the build)
+    even = _sums_batch(np.full(len(sizes), sizes.sum() // len(sizes)))[-1]
+    assert ms[0] <= 6.0 * even[0]
+    assert ms[1] <= 2.0 * even[1]
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
