@@ -118,11 +118,12 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 
 __device__ __forceinline__ void set_status(int* status, int bits) { atomicOr(status, bits); }
 
-// 1 / sqrt(x) to about an ulp in three FP64 instructions where the library
-// takes ten: the FP32 estimate y with its FP64 remainder e = 1 - x y^2
-// (|e| < 2^-20), y (1 + e/2 + 3/8 e^2) with the last term (below 2^-41)
-// formed in FP32 and placed in the 29 low bits that y leaves free, and the
-// conversions done on the bit patterns.  x in [2^-120, 2^120].
+// 1 / sqrt(x) to an ulp in three FP64 instructions where the library takes ten:
+// the FP32 estimate y with its FP64 remainder e = 1 - x y^2 (y^2 is exact, |e| <
+// 2^-21) and the Taylor series of y / sqrt(1 - e) to second order, y (1 + e/2 +
+// 3/8 e^2), with the last term (below 2^-43) formed in FP32 and placed in the 29
+// low bits that y leaves free, and the conversions done on the bit patterns.
+// x in [2^-120, 2^120].
 __device__ __forceinline__ double rsqrt_refined(double x) {
   const unsigned hi = __double2hiint(x), lo = __double2loint(x);
   float y;
@@ -130,7 +131,7 @@ __device__ __forceinline__ double rsqrt_refined(double x) {
   const unsigned yb = __float_as_uint(y);
   const unsigned yh = (yb >> 3) + 0x38000000u, yl = yb << 29;
   const double yd = __hiloint2double(yh, yl);
-  const double e = fma(-(x * yd), yd, 1.0);
+  const double e = fma(-x, yd * yd, 1.0);
   const float ef = __int_as_float(max((__double2hiint(e) & 0x7fffffff) - 0x38000000, 0) << 3);
   const float k = (0.375f * 0x1p52f) * (ef * ef) * __uint_as_float((yb & 0x7fffffu) | 0x3f800000u);
   const unsigned n = __float_as_uint(k + 8388608.0f) & 0x7fffffu;  // k rounded to an integer (< 2^12)
