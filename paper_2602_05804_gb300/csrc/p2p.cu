@@ -665,7 +665,10 @@ __global__ void k_p2p_combine(const P2PArgs a) {
   }
 }
 
+// Blocks per SM that fit, asked once per context (a query takes the host about
+// as long as a launch).
 int p2p_blocks_fit(sfmm_ctx* c) {
+  if (c->p2p_fit > 0) return c->p2p_fit;
   int per_sm = 0;
   if (c->precision == SFMM_FP32) {
     const int smem = P2P_WARPS * (int)sizeof(P2PWarp);
@@ -673,8 +676,9 @@ int p2p_blocks_fit(sfmm_ctx* c) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_f32, P2P_NT, smem);
   } else {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p_fexp, FX_NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->p2p_fit64, k_p2p_fp64, P64_NT, 0);
   }
-  return per_sm < 1 ? 1 : per_sm;
+  return c->p2p_fit = per_sm < 1 ? 1 : per_sm;
 }
 
 int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
@@ -786,8 +790,7 @@ int run_p2p(sfmm_ctx* c, double* acc, double* pot) {
     k_p2p_fexp<<<nblocks, FX_NT, 0, c->stream>>>(a, f);
     a.leaf_counter = f.fb + 1;
     a.items = f.fb + 4;
-    int fit64 = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit64, k_p2p_fp64, P64_NT, 0);
+    int fit64 = c->p2p_fit64;
     if (c->p2p_blocks > 0 && c->p2p_blocks < fit64) fit64 = c->p2p_blocks;
     k_p2p_fp64<<<std::max(1, fit64) * num_sms(c->device), P64_NT, 0, c->stream>>>(a);
     c->nlaunch += 2;

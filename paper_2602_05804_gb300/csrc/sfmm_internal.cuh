@@ -71,6 +71,7 @@ struct sfmm_ctx {
   int schedule = 0;         // walk mode 1: 0 automatic, 1 one launch per depth, 2 readiness queue
   int p2p_chunk = SFMM_P2P_CHUNK_DEFAULT;  // most neighbour-list entries per near-field work item
   int p2p_blocks = 0;       // near-field blocks per SM (0: as many as fit)
+  int p2p_fit = 0, p2p_fit64 = 0;  // blocks per SM that fit: the form's near field, the FP64 kernel's (0: not asked yet)
   int max_depth = 0;
   std::vector<int> h_level_off;  // host copy: internal nodes per depth, max_depth + 2 entries
   int* h_level_pin = nullptr;     // pinned landing buffer of the level offsets (and their total)
