@@ -26,13 +26,14 @@
 // holds at most 1/12 of all (10^6 particles: 1.87 ms; 1/4 1.89, 1/8 1.88, 1/16
 // 1.90, own marks always 1.89, dealt always 1.98).
 #define P2P_OWN 12
-// Where 2 h_max of the leaf is beyond three times its size, about half of the
-// candidates lie inside a kernel and all of them are evaluated with both
+// Where 2h of every target is beyond three times the leaf's size, about half of
+// the candidates lie inside a kernel and all of them are evaluated with both
 // kernels at once, without the unsoftened pass (uniform set of 3 10^5 with h of
 // 2, 3, 4, 6, 12 mean spacings, this line, never, and always the dealt marks:
-// 1.00 1.01 1.24, 2.25 2.49 3.46, 4.12 4.83 7.45, 10.1 12.7 22.0, 50.6 68.1 137
-// ms; line at 2: 10^5 particles at order 4 0.377 instead of 0.341 ms, at 4 the
-// 3-spacing set 2.39, at 6 2.48 ms).
+// 1.00 1.01 1.24, 2.29 2.49 3.46, 4.17 4.83 7.45, 10.3 12.7 22.0, 51.7 68.1 137
+// ms; the line at 2: 1.03 for the first, at 4: 2.41 for the second.  By the
+// largest 2h a leaf at a binary's surface, with one wide kernel among narrow
+// ones, would take this path: leaves of 48, theta 0.4: 1.85 instead of 1.76 ms).
 #define P2P_DENSE 3.0f
 struct P2PWarp {
   float4 far[P2P_SB];   // pairs, negated: [q/2] {x0, x1, y0, y1}, [SB/2 + q/2] {z0, z1, m0, m1}
@@ -89,7 +90,6 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
     const float4 hiL = a.geo_hi[L], loL = a.geo_lo[L];
     const float lL = hiL.w * 1.0001f;
     const float hL = loL.w * 1.0001f;
-    const bool dense = 2.0f * hL > P2P_DENSE * lL;
     // lane -> (target slot, phase); more than 32 targets: a second slot, 32 on
     const int nph = (nL <= 16) ? (32 / nL) : 1;
     const int ntl = (nL <= 32) ? nL : 32;
@@ -115,6 +115,9 @@ __global__ void __launch_bounds__(P2P_NT, 4) k_p2p_f32(const P2PArgs a) {
     };
     float xi, yi, zi, h2i;
     load_targets(0, xi, yi, zi, h2i);
+    // least (2h)^2 of the (first 32) targets, as bits
+    const unsigned h2m = __reduce_min_sync(SFMM_FULL, __float_as_uint(lane_on && t0 < nL ? h2i : INFINITY));
+    const bool dense = __uint_as_float(h2m) > (P2P_DENSE * P2P_DENSE) * (lL * lL);
     float ax = 0.0f, ay = 0.0f, az = 0.0f, pt = 0.0f;      // current slot
     float bx = 0.0f, by = 0.0f, bz = 0.0f, bp = 0.0f;      // the other one
 
