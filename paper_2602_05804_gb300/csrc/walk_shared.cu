@@ -209,8 +209,8 @@ __device__ __forceinline__ void leaf_l2p(const LevelArgs& la, int A, double cAx,
 #include "walk_pair.cuh"
 
 // Blocks per SM (FP32, p <= 2): 5 for the queue walk, 4 per depth -- measured:
-// the queue walk gains from the fifth block despite a few spilled registers,
-// the per-depth walk loses.
+// the queue walk gains from the fifth block (96 registers, none spilled now that
+// an interaction keeps 19 sums), the per-depth walk (114 registers) loses.
 template <int P, bool F32, bool SYM, bool QUEUE>
 __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? (QUEUE ? 5 : 4) : 1) k_walk_level(const LevelArgs la) {
   static_assert(!(SYM && QUEUE), "the queue walk runs walk mode 1 only");
@@ -920,7 +920,10 @@ static int run_levels(sfmm_ctx* c, double theta, int order) {
 // Capacity overflow of the shared walk (status bits of the last run, its
 // counters in hs): grow what ran out before the rerun.
 int walk_shared_regrow(sfmm_ctx* c, int bits, const unsigned long long* hs) {
-  if (bits & SFMM_ST_RING) c->ring_capacity = c->ring_capacity < (1 << 20) ? c->ring_capacity * 16 : (1 << 24);
+  // (sixteen-fold once, then four-fold: the rings of the pair walk's 3040 warps
+  // take 10 GB at 2^17 entries, 43 at 2^19 and 172 at 2^21)
+  if (bits & SFMM_ST_RING)
+    c->ring_capacity = std::min(1 << 24, c->ring_capacity * (c->ring_capacity < (1 << 17) ? 16 : 4));
   if (bits & SFMM_ST_ARENA) {
     const unsigned long long need = hs[9];
     const int64_t grown = 2 * c->walk_arena_cap, want = (int64_t)(need + need / 4 + 1024);

@@ -1,7 +1,8 @@
 """Paths that small sets and batches take: the one-block sort and scan at the
-edges of their ranges (4096 particles, 8192 values), sums over slices of 8192
-particles of a system, neighbour lists cut finer than the option when the lists
-are few, and FP64 moments translated a moment per lane where few lanes climb."""
+edges of their ranges (4096 particles, 8192 values), sums and boxes over slices
+of a batch's systems, neighbour lists cut finer than the option when the lists
+are few, FP64 moments translated a moment per lane where few lanes climb, and
+the device memory that small sets and long lists take."""
 import math
 
 import numpy as np
@@ -196,3 +197,26 @@ def test_moments_of_the_climb(order, n, leaf):
     for k, deg in enumerate(np.asarray(mi).sum(1)):
         scale = t["mass"] * (t["size"] + 1e-16) ** deg + (1e-15 * t["mass"] if deg == 1 else 0.0)
         assert (np.abs(Q[:, k] - Qr[:, k]) <= 1e-14 * scale + 1e-30).all(), (order, k)
+
+
+def test_walk_rings_grow_by_what_a_long_list_needs():
+    """One kernel wider than the set: its leaf opens every other one, a list of
+    more than 2^17 entries.  The rings of all resident warps then grow to 2^19
+    entries (43 GB in the pair walk), not to 2^21 (172 GB)."""
+    import torch
+
+    pos, m, h = workloads.plummer(600_000, 6)
+    h = h.copy()
+    h[0] = 30.0
+    pos, m, h = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (pos, m, h))
+    torch.cuda.synchronize()
+    got = []
+    for sched in (3, 2):
+        free = torch.cuda.mem_get_info()[0]
+        s = solver("fp32", schedule=sched)
+        s.build(pos, m, h, 4)
+        got.append([t.cpu().numpy() for t in s.gravity(0.7, 1)])
+        assert free - torch.cuda.mem_get_info()[0] <= 60e9
+        s.close()
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    np.testing.assert_array_equal(got[0][1], got[1][1])
