@@ -836,7 +836,7 @@ def run_gpu(args):
         nm2l = st32["m2l_unique"] if args.walk >= 1 else st32["m2l"]
         kname = "k_walk_level<2,FP32>" if args.walk >= 1 else "k_walk<2,FP32>"
         kms = st32["ms_walk"]
-        achieved = nm2l * 136 / (kms * 1e-3) / 1e12
+        achieved = nm2l * M2L_FLOPS_P2 / (kms * 1e-3) / 1e12
         src = _kernel_hash("walk_shared.cu" if args.walk >= 1 else "walk.cu", "walk_common.cuh", "expansion_gen.cuh")
     roof = {"kernel": kname, "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
             "frac": achieved / fp32_peak, "traffic": _traffic(kname, src),

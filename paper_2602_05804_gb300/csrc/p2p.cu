@@ -70,8 +70,9 @@ struct P2PArgs {
 // Neighbour-list entries per work item: the option's value, fewer when the
 // lists are too few for eight items per resident warp, down to p2p_chunk_least.
 // With 256 entries throughout, the near field of 1000 particles took 54 us in
-// 96 items and that of a binary of 13,000 in the FP64 form (several calls of a
-// leapfrog run) 4.9 ms in 2500 items on 2432 warps; 32 us and 2.0 ms cut finer.
+// 96 items and that of a binary of 13,000 in the FP64 form, after eight leapfrog
+// steps of its collapse (5.1e7 pairs), 4.9 ms in 2500 items on 2432 warps; 32 us
+// and 2.0 ms cut finer.
 __device__ __forceinline__ int p2p_chunk_of(unsigned long long total, int most, int least, int want) {
   const unsigned long long c = total / (unsigned)want;
   return c >= (unsigned long long)most ? most : max(least, (int)c);
@@ -136,7 +137,8 @@ __device__ __forceinline__ float rsqrt_normal(float x) {
 
 // Two unsoftened pairs of one target in the packed FP32 instructions (two
 // lanes of FP32 per register pair, one issue slot): sources given negated,
-// (-x, -y, -z, -m), so that every operation rounds exactly as pair_far's.
+// (-x, -y, -z, -m), so that every operation rounds as the scalar one on the
+// values themselves.
 __device__ __forceinline__ void pair_far2(float2 xi, float2 yi, float2 zi, float2 nx, float2 ny, float2 nz,
                                           float2 nm, float2& ax, float2& ay, float2& az, float2& pt) {
   const float2 dx = __fadd2_rn(xi, nx), dy = __fadd2_rn(yi, ny), dz = __fadd2_rn(zi, nz);

@@ -18,13 +18,15 @@
 // candidate, the whole warp ran them for almost every step, because some lane
 // nearly always is inside a kernel: the candidates took 122 issue cycles per
 // 32 pairs where the unsoftened sources take 23.  Measured, in place and now:
-// 2.25 and 1.86 ms for the 1.38e9 pairs of a Plummer sphere of 10^6, 7.58 and
-// 6.37 ms at theta 0.3, 34.5 and 28.4 ms for a clustered cloud of 1.6e7.
+// 2.25 and 1.87 ms for the 1.38e9 pairs of a Plummer sphere of 10^6 (0.82 of the
+// issue slots, 25 of 32 lanes), 7.58 and 6.43 ms at theta 0.3, 34.5 and 28.5 ms
+// for a clustered cloud of 1.6e7.  Without the dealt marks (less code) leaves of
+// 16 gain 1 % and leaves of 24 and more lose 2 to 5 %.
 #define P2P_RES 64  // marked pairs evaluated before their owners collect
-// A group of 32 dealt marks takes about twelve times a mark evaluated by its
-// own lane takes from a warp's lane share: own marks where the fullest lane
-// holds at most 1/12 of all (10^6 particles: 1.87 ms; 1/4 1.89, 1/8 1.88, 1/16
-// 1.90, own marks always 1.89, dealt always 1.98).
+// Own marks take as many steps as the fullest lane has, dealt ones a 32nd of all
+// marks at about four times a step.  Own marks where the fullest lane holds at
+// most 1/12 of all (10^6 particles: 1.87 ms; 1/4 1.89, 1/8 1.88, 1/16 1.90, own
+// marks always 1.89, dealt always 1.98).
 #define P2P_OWN 12
 // Where 2h of every target is beyond three times the leaf's size, about half of
 // the candidates lie inside a kernel and all of them are evaluated with both

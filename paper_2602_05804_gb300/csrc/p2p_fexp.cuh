@@ -7,8 +7,9 @@
 // FP32 pipe, and the FP64 pipe only evaluates the softened pairs, 32 at a time
 // with every lane busy, while other warps of the SM quarter run expansions.
 // Measured, before and now: 66.6 and 17.5 ms for the 1.38e9 pairs of a Plummer
-// sphere of 10^6 (FMA pipe 64 % busy, FP64 40 %; 16 warps per SM by registers
-// and shared memory: 19.0 ms with twenty, 18.7 with twelve), 5.87 and 1.75 ms
+// sphere of 10^6 (FMA pipe 64 % busy, FP64 40 %; 16 warps per SM by shared
+// memory and 128 registers, of which 140 bytes are spilled: 19.0 ms with twenty,
+// 18.7 with twelve), 5.87 and 1.75 ms
 // for 10^5 with leaves of 8, 0.77 and 0.23 ms for 10^4 (the last two with the
 // finer list chunks).
 //
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(FX_NT, 4) k_p2p_fexp(const P2PArgs a, const Fe
         e += 32;
       }
       if (stream_left) {
-        // stage one window of up to 32 particles of the stream (as k_p2p)
+        // stage one window of up to 32 particles of the stream (as k_p2p_f32)
         const int p = pdone + lane;
         const bool valid = p < tot;
         const bool pre = cum < pdone;

@@ -1166,14 +1166,7 @@ __device__ __forceinline__ void upward_node(int v, int R, double* ncx, double* n
   }
 }
 
-// Bottom-up: the second child to finish computes its parent.  The climb's
-// cost is its longest chain of dependent arrivals (one device-scope fence,
-// atomic and round of loads per level: about 30 levels on a Plummer sphere
-// of 10^6), so the node body issues all its loads at once.  (Measured on
-// GB300: computing the top of the tree -- the ~1500 nodes of more than 10^3
-// particles, 23 levels deep -- level by level in one block after a climb
-// that stops below it was slower, 0.18 against 0.13 ms.)
-// The climb with FP64 moments, warp by warp.  An FP64 instruction takes the
+// The climb (k_upward, below) with FP64 moments, warp by warp.  An FP64 instruction takes the
 // pipe about 80 cycles whatever the active lanes, and near the top of the tree
 // one or two lanes of a warp climb: up to four of them have their moments
 // translated one node after the other by the whole warp, a moment per lane (12
@@ -1278,6 +1271,13 @@ __global__ void __launch_bounds__(128) k_upward_fp64(const uint32_t* __restrict_
   }
 }
 
+// Bottom-up: the second child to finish computes its parent.  The climb's
+// cost is its longest chain of dependent arrivals (one device-scope fence,
+// atomic and round of loads per level: about 30 levels on a Plummer sphere
+// of 10^6), so the node body issues all its loads at once.  (Measured on
+// GB300: computing the top of the tree -- the ~1500 nodes of more than 10^3
+// particles, 23 levels deep -- level by level in one block after a climb
+// that stops below it was slower, 0.18 against 0.13 ms.)
 template <int P, typename QT>
 __global__ void k_upward(const uint32_t* __restrict__ counts, const int* __restrict__ leaf_node, const int* __restrict__ nparent,
                          const int* __restrict__ nright, double* ncx, double* ncy, double* ncz, double* nmass,

@@ -89,7 +89,8 @@ __device__ __forceinline__ void pair_decide(PairKid& k, int s, const float4& hiB
 
 
 // Five blocks per SM (96 registers, 64 bytes spilled): 14.7 ms on the 1.6e7
-// cloud, four (128 registers) 16.0, six 15.2.
+// cloud, four (128 registers) 16.0, six 15.2 (before the branch-free acceptance
+// test; 13.8 with it).
 template <int P, bool F32>
 __global__ void __launch_bounds__(WALK_NT, (P <= 2 && F32) ? 5 : 1) k_walk_pair(const LevelArgs la) {
   using E = Exp<P>;

@@ -279,7 +279,10 @@ class Solver:
     """One context: ``build`` then ``gravity`` on torch CUDA float64 tensors.
 
     precision: "fp64" or "fp32" (the FP32 form).  Work is issued on the
-    current torch stream of the device at creation time (or ``stream``).
+    current torch stream of the device at creation time (or ``stream``); where
+    that is torch's default stream, on a stream of the solver's own, which does
+    not wait for work queued on the default one: arrays passed in have to be
+    complete.  Every call returns after its own work has completed.
     """
 
     def __init__(self, device: int = 0, precision: str = "fp32", stream=None, **options):
